@@ -71,6 +71,7 @@ void free_all(g4_ctx* h) {
     xtc_release(h);
     nfft_release(h);
     direct_release(h);
+    f64tc_release(h);
     void* ptrs[] = {h->kadd, h->ksub, h->acc, h->dstatus, h->Gfull, h->Gd, h->pairs, h->hstage};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -115,15 +116,23 @@ g4_status sync_and_check(g4_ctx* h) {
     return check_status(h);
 }
 
+// The batch's update: on tensor cores where the handle has that plan and the
+// batch is large enough (the plain kernels then run only if the batch's flag
+// is set), else by the plain kernels.
 g4_status accumulate_fp64(g4_ctx* h) {
-    const size_t NN = (size_t)h->d.N * h->d.N;
-    for (int r = 0; r < h->staged; ++r) {
-        prof_begin(h, G4_K_UPDATE_FP64);
-        cudaError_t e = launch_update_fp64(h->Gfull + (size_t)r * 2 * NN, h->slot_sign[r], h->acc,
-                                           h->kadd, h->ksub, h->d, h->stream);
-        prof_end(h, G4_K_UPDATE_FP64);
-        if (e != cudaSuccess) return g4_cuda_fail(h, e, "update_fp64 launch");
+    G4Signs signs;
+    for (int r = 0; r < h->staged; ++r) signs.s[r] = h->slot_sign[r];
+    const unsigned* only_if = nullptr;
+    if (f64tc_wanted(h, h->staged)) {
+        g4_status st = f64tc_run(h, h->staged);
+        if (st != G4_OK) return st;
+        only_if = h->gmax;
     }
+    prof_begin(h, G4_K_UPDATE_FP64);
+    cudaError_t e = launch_update_fp64(h->Gfull, signs, h->staged, h->acc, h->kadd, h->ksub, h->d,
+                                       only_if, h->stream);
+    prof_end(h, G4_K_UPDATE_FP64);
+    if (e != cudaSuccess) return g4_cuda_fail(h, e, "update_fp64 launch");
     return G4_OK;
 }
 
@@ -182,9 +191,11 @@ g4_status stage_measurement(g4_ctx* h, const void* M, bool m64, const void* G0, 
         h->slots->s[slot] = G4Slot{M, (const double2*)G0, f.rs, f.neg ? 1 : 0};
     } else if (h->opt.precision == G4_PREC_FP64) {
         const size_t NN = (size_t)h->d.N * h->d.N;
+        if (slot == 0 && h->f64tc) e = cudaMemsetAsync(h->gmax, 0, sizeof(unsigned), h->stream);
         prof_begin(h, G4_K_BUILD_G);
-        e = launch_build_G_fp64(M, m64, (const double2*)G0, h->Gfull + (size_t)slot * 2 * NN,
-                                h->d.N, h->stream);
+        if (e == cudaSuccess)
+            e = launch_build_G_fp64(M, m64, (const double2*)G0, h->Gfull + (size_t)slot * 2 * NN,
+                                    h->d.N, h->f64tc ? h->gmax : nullptr, h->stream);
         prof_end(h, G4_K_BUILD_G);
     } else {
         // the largest |G~| of the batch starts again with its first measurement
@@ -394,6 +405,7 @@ g4_status g4_create(int Nc, int Nw, int Nwex, int Nkex, g4_channel ch, const g4_
         }
         if (has_direct(d.ch) && (st = direct_prepare(h)) != G4_OK) return fail(st);
     }
+    if (opt.precision == G4_PREC_FP64) f64tc_prepare(h);
     if ((st = g4_reset(h)) != G4_OK) return fail(st);
     ce = cudaStreamSynchronize(h->stream);
     if (ce != cudaSuccess) {
@@ -798,7 +810,7 @@ void g4_destroy(g4_handle h) {
 
 g4_status g4_build_G(int N, const void* M, const void* G0, void* G, void* stream) {
     if (N < 1 || !M || !G0 || !G) return g4_fail(nullptr, G4_ERR_INVALID, "bad g4_build_G arguments");
-    cudaError_t e = launch_build_G_fp64(M, false, (const double2*)G0, (double2*)G, N,
+    cudaError_t e = launch_build_G_fp64(M, false, (const double2*)G0, (double2*)G, N, nullptr,
                                         (cudaStream_t)stream);
     if (e != cudaSuccess) return g4_cuda_fail(nullptr, e, "build_G launch");
     return G4_OK;

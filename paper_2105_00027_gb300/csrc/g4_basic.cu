@@ -6,6 +6,7 @@
 //     (the accumulation of Eq. (1), Sec. 2.1);
 //   * the final normalisation by the sign sum and the transpose to the
 //     exported layout.
+#include <algorithm>
 #include <type_traits>
 
 #include "g4_gtilde.cuh"
@@ -18,126 +19,169 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
     return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-template <bool M64>
-__device__ __forceinline__ double2 load_m(const void* M, size_t i) {
-    if (M64) {
-        float2 v = reinterpret_cast<const float2*>(M)[i];
-        return make_double2(v.x, v.y);
-    } else {
-        return reinterpret_cast<const double2*>(M)[i];
-    }
-}
+// G[sp][i][j] = G0[sp][i] d_ij - G0[sp][i] M[sp][i][j] G0[sp][j], FP64.  A
+// block takes kBuildU blocks of columns of one row (no division per entry,
+// kBuildU independent loads in flight); flag (may be null): see
+// launch_build_G_fp64, tested on the exponent fields.
+constexpr int kBuildU = 4;
 
-// G[sp][i][j] = G0[sp][i] d_ij - G0[sp][i] M[sp][i][j] G0[sp][j], FP64.
 template <bool M64>
-__global__ void k_build_G_fp64(const void* __restrict__ M, const double2* __restrict__ G0,
-                               double2* __restrict__ G, int N) {
-    const size_t NN = (size_t)N * N;
-    const size_t total = 2 * NN;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
-         e += (size_t)gridDim.x * blockDim.x) {
-        const int sp = (int)(e / NN);
-        const size_t ij = e - (size_t)sp * NN;
-        const int i = (int)(ij / N), j = (int)(ij - (size_t)i * N);
-        const double2 gi = G0[sp * N + i], gj = G0[sp * N + j];
-        double2 v = cmul(cmul(gi, load_m<M64>(M, e)), gj);
-        v.x = -v.x;
-        v.y = -v.y;
-        if (i == j) {
-            v.x += gi.x;
-            v.y += gi.y;
+__global__ void __launch_bounds__(256) k_build_G_fp64(const void* __restrict__ M,
+                                                      const double2* __restrict__ G0,
+                                                      double2* __restrict__ G, int N,
+                                                      unsigned* __restrict__ flag) {
+    using MV = typename std::conditional<M64, float2, double2>::type;
+    bool bad = false;
+    const int j0 = blockIdx.x * (kBuildU * blockDim.x) + threadIdx.x;
+    for (int row = blockIdx.y; row < 2 * N; row += gridDim.y) {
+        const int sp = row >= N ? 1 : 0, i = row - sp * N;
+        const double2 gi = G0[row], ngi = make_double2(-gi.x, -gi.y);
+        const MV* mrow = reinterpret_cast<const MV*>(M) + (size_t)row * N;
+        MV m[kBuildU];
+        double2 gj[kBuildU];
+#pragma unroll
+        for (int u = 0; u < kBuildU; ++u) {
+            const int j = j0 + u * blockDim.x;
+            if (j < N) {
+                m[u] = mrow[j];
+                gj[u] = G0[sp * N + j];
+            }
         }
-        G[e] = v;
+#pragma unroll
+        for (int u = 0; u < kBuildU; ++u) {
+            const int j = j0 + u * blockDim.x;
+            if (j >= N) break;
+            double2 v = cmul(cmul(ngi, make_double2(m[u].x, m[u].y)), gj[u]);
+            if (i == j) v = make_double2(v.x + gi.x, v.y + gi.y);
+            G[(size_t)row * N + j] = v;
+            // on the exponent fields, off the FP64 pipe (which bounds this kernel)
+            const long long bx = __double_as_longlong(v.x) & 0x7FFFFFFFFFFFFFFFll;
+            const long long by = __double_as_longlong(v.y) & 0x7FFFFFFFFFFFFFFFll;
+            constexpr unsigned lo = (unsigned)(1023 - kF64tcExp) << 20, span = (unsigned)(2 * kF64tcExp) << 20;
+            bad = bad || ((unsigned)(bx >> 32) - lo > span && bx != 0) ||
+                  ((unsigned)(by >> 32) - lo > span && by != 0);
+        }
     }
+    if (flag && bad) *flag = 1u;
 }
 
-// One measurement's FP64 update of every accumulator entry, for channel CH
-// (see g4.h).  Block row K1 = blockIdx.y; threads run over (K2, Q) with Q
-// fastest, so the accumulator read-modify-write is coalesced.
-template <int CH>
-__global__ void k_update_fp64(const double2* __restrict__ G, double sign,
-                              double2* __restrict__ acc, const int* __restrict__ kadd,
-                              const int* __restrict__ ksub, G4Dims d) {
+// The staged measurements' FP64 update of every accumulator entry, for channel
+// CH (see g4.h).  Block row K1 = blockIdx.y; groups of RS lanes run over (K2, Q)
+// with Q fastest, so the accumulator read-modify-write, once per batch, is
+// coalesced; the lanes of a group share out the measurements and add up their
+// sums by shuffles.  The kernel of shapes the tiled one does not take (RS = 1)
+// and of small problems, where a lane's chain over the measurements is the
+// whole time (1024 entries, 16 measurements: 29 us with RS = 1, 5 with 16).
+template <int CH, int RS>
+__global__ void k_update_fp64(const double2* __restrict__ Gb, const __grid_constant__ G4Signs signs,
+                              int staged, double2* __restrict__ acc, const int* __restrict__ kadd,
+                              const int* __restrict__ ksub, G4Dims d,
+                              const unsigned* __restrict__ only_if) {
+    if (only_if && !*only_if) return;
     const int K1 = blockIdx.y;
     const int k1 = K1 / d.Nw2, n1 = K1 - k1 * d.Nw2;
     const size_t NN = (size_t)d.N * d.N;
     const int per = d.N * d.NQ;
     double2* row = acc + (size_t)K1 * per;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < per;
-         idx += gridDim.x * blockDim.x) {
+    const int sub = threadIdx.x % RS, step = gridDim.x * (blockDim.x / RS);
+    // a warp's lanes stay together to the end (the shuffles take all of them)
+    const int first = blockIdx.x * (blockDim.x / RS) + threadIdx.x / RS;
+    for (int base = first - (int)(threadIdx.x & 31) / RS; base < per; base += step) {
+        const int idx0 = base + (int)(threadIdx.x & 31) / RS, idx = min(idx0, per - 1);
         const int K2 = idx / d.NQ, Qi = idx - K2 * d.NQ;
         const int q = Qi / d.Nwex, m = d.m0 + Qi - q * d.Nwex;   // m: the transfer frequency
         const int k2 = K2 / d.Nw2, n2 = K2 - k2 * d.Nw2;
-        double2 term = make_double2(0, 0);
-        if (CH == G4_PP_UPDOWN) {
-            // G_s(Q-K2, Q-K1) G_-s(K2, K1); Q-K has frequency index m + Nw2-1 - n
-            const int f1 = m + d.Nw2 - 1 - n1, f2 = m + d.Nw2 - 1 - n2;
-            if (f1 >= 0 && f1 < d.Nw2 && f2 >= 0 && f2 < d.Nw2) {
-                const int QK1 = ksub[q * d.Nc + k1] * d.Nw2 + f1;
-                const int QK2 = ksub[q * d.Nc + k2] * d.Nw2 + f2;
+        double2 o = make_double2(0.0, 0.0);
+        for (int r = sub; r < staged; r += RS) {
+            const double2* G = Gb + (size_t)(2 * r) * NN;
+            const double sign = signs.s[r];
+            double2 term = make_double2(0, 0);
+            if (CH == G4_PP_UPDOWN) {
+                // G_s(Q-K2, Q-K1) G_-s(K2, K1); Q-K has frequency index m + Nw2-1 - n
+                const int f1 = m + d.Nw2 - 1 - n1, f2 = m + d.Nw2 - 1 - n2;
+                if (f1 >= 0 && f1 < d.Nw2 && f2 >= 0 && f2 < d.Nw2) {
+                    const int QK1 = ksub[q * d.Nc + k1] * d.Nw2 + f1;
+                    const int QK2 = ksub[q * d.Nc + k2] * d.Nw2 + f2;
+#pragma unroll
+                    for (int sp = 0; sp < 2; ++sp) {
+                        const double2 t = cmul(G[sp * NN + (size_t)QK2 * d.N + QK1],
+                                               G[(1 - sp) * NN + (size_t)K2 * d.N + K1]);
+                        term.x += t.x;
+                        term.y += t.y;
+                    }
+                }
+            } else {
+                const bool v1 = n1 + m < d.Nw2, v2 = n2 + m < d.Nw2;
+                const int K1Q = kadd[k1 * d.Nc + q] * d.Nw2 + n1 + m;
+                const int K2Q = kadd[k2 * d.Nc + q] * d.Nw2 + n2 + m;
+                double2 a = make_double2(0, 0), b = make_double2(0, 0), ex = make_double2(0, 0);
 #pragma unroll
                 for (int sp = 0; sp < 2; ++sp) {
-                    const double2 t = cmul(G[sp * NN + (size_t)QK2 * d.N + QK1],
-                                           G[(1 - sp) * NN + (size_t)K2 * d.N + K1]);
-                    term.x += t.x;
-                    term.y += t.y;
-                }
-            }
-        } else {
-            const bool v1 = n1 + m < d.Nw2, v2 = n2 + m < d.Nw2;
-            const int K1Q = kadd[k1 * d.Nc + q] * d.Nw2 + n1 + m;
-            const int K2Q = kadd[k2 * d.Nc + q] * d.Nw2 + n2 + m;
-            double2 a = make_double2(0, 0), b = make_double2(0, 0), ex = make_double2(0, 0);
-#pragma unroll
-            for (int sp = 0; sp < 2; ++sp) {
-                const double2* g = G + sp * NN;
-                const double wgt = (CH == G4_PH_MAGNETIC && sp) ? -1.0 : 1.0;
-                if (CH != G4_PH_TRANSVERSE) {
-                    if (v1) {
-                        const double2 t = g[(size_t)K1Q * d.N + K1];
-                        a.x += wgt * t.x;
-                        a.y += wgt * t.y;
+                    const double2* g = G + sp * NN;
+                    const double wgt = (CH == G4_PH_MAGNETIC && sp) ? -1.0 : 1.0;
+                    if (CH != G4_PH_TRANSVERSE) {
+                        if (v1) {
+                            const double2 t = g[(size_t)K1Q * d.N + K1];
+                            a.x += wgt * t.x;
+                            a.y += wgt * t.y;
+                        }
+                        if (v2) {
+                            const double2 t = g[(size_t)K2 * d.N + K2Q];
+                            b.x += wgt * t.x;
+                            b.y += wgt * t.y;
+                        }
                     }
-                    if (v2) {
-                        const double2 t = g[(size_t)K2 * d.N + K2Q];
-                        b.x += wgt * t.x;
-                        b.y += wgt * t.y;
+                    if (v1 && v2) {
+                        // transverse pairs the opposite spin in the G(K2,K1) factor
+                        const double2* gx = CH == G4_PH_TRANSVERSE ? G + (1 - sp) * NN : g;
+                        const double2 t = cmul(gx[(size_t)K2 * d.N + K1], g[(size_t)K1Q * d.N + K2Q]);
+                        ex.x += t.x;
+                        ex.y += t.y;
                     }
                 }
-                if (v1 && v2) {
-                    // transverse pairs the opposite spin in the G(K2,K1) factor
-                    const double2* gx = CH == G4_PH_TRANSVERSE ? G + (1 - sp) * NN : g;
-                    const double2 t = cmul(gx[(size_t)K2 * d.N + K1], g[(size_t)K1Q * d.N + K2Q]);
-                    ex.x += t.x;
-                    ex.y += t.y;
-                }
+                const double2 ab = cmul(a, b);
+                term = make_double2(ab.x - ex.x, ab.y - ex.y);
             }
-            const double2 ab = cmul(a, b);
-            term = make_double2(ab.x - ex.x, ab.y - ex.y);
+            o.x += sign * term.x;
+            o.y += sign * term.y;
         }
-        double2 o = row[idx];
-        o.x += sign * term.x;
-        o.y += sign * term.y;
-        row[idx] = o;
+#pragma unroll
+        for (int w = RS / 2; w > 0; w >>= 1) {
+            o.x += __shfl_xor_sync(0xffffffffu, o.x, w);
+            o.y += __shfl_xor_sync(0xffffffffu, o.y, w);
+        }
+        if (sub == 0 && idx0 < per) row[idx] = make_double2(row[idx].x + o.x, row[idx].y + o.y);
     }
 }
 
 // The same FP64 update for the particle-hole channels, tiled: a block owns a
 // momentum pair (k1, k2) and a 16 x 16 tile of frequencies (n1, n2), one thread
-// per (n1, n2), and walks the transfer momenta q.  For each q it stages in
-// shared memory what the tile's products read -- the window of the G blocks
-// (k1 (+) q, k2 (+) q) at rows n1 + m and columns n2 + m (exchange factor), the
-// spin-weighted band G(K1+Q, K1) (a) and G(K2, K2+Q) (b) -- next to the fixed
-// G(K2, K1) tile, and each thread adds its Nwex transfers m, so that over the
-// q walk a thread updates its entries acc[K1][K2][q][m] in order (every line of
-// the accumulator written whole).  Nwex <= kTileWex.
+// per (n1, n2), and walks the transfer momenta q and, inside, the staged
+// measurements.  For each it stages in shared memory what the tile's products
+// read -- the window of the G blocks (k1 (+) q, k2 (+) q) at rows n1 + m and
+// columns n2 + m (exchange factor), the spin-weighted band G(K1+Q, K1) (a) and
+// G(K2, K2+Q) (b), the G(K2, K1) tile -- and each thread sums its Nwex <= WX
+// transfers in registers: the accumulator is read and written once per batch,
+// and the sign rides on a and the G(K2, K1) tile, so that an element-update is
+// twelve fused multiply-adds.  Bound by the FP64 pipe (two lanes per clock and
+// SM): per-measurement launches of eighteen operations per update ran at
+// 3.0e10 updates/s on the 4x4 cluster with 64 frequencies.
 constexpr int kTileF = 16;      // frequencies per tile side
 constexpr int kTileWex = 16;    // largest Nwex of the tiled form
 
-template <int CH>
+__device__ __forceinline__ void cfma(double2& t, double2 a, double2 b) {
+    t.x = fma(a.x, b.x, t.x);
+    t.y = fma(a.x, b.y, t.y);
+    t.x = fma(-a.y, b.y, t.x);
+    t.y = fma(a.y, b.x, t.y);
+}
+
+template <int CH, int WXM>
 __global__ void __launch_bounds__(kTileF * kTileF) k_update_fp64_tiled(
-    const double2* __restrict__ G, double sign, double2* __restrict__ acc,
-    const int* __restrict__ kadd, G4Dims d) {
+    const double2* __restrict__ Gb, const __grid_constant__ G4Signs signs, int staged,
+    double2* __restrict__ acc, const int* __restrict__ kadd, G4Dims d,
+    const unsigned* __restrict__ only_if) {
+    if (only_if && !*only_if) return;
     extern __shared__ double2 sm[];
     const int Nw2 = d.Nw2, N = d.N, Nwex = d.Nwex;
     const int nt = (Nw2 + kTileF - 1) / kTileF;
@@ -153,71 +197,72 @@ __global__ void __launch_bounds__(kTileF * kTileF) k_update_fp64_tiled(
     double2* A = X1 + 2 * kTileF * (kTileF + 1);     // [kTileF t1][Nwex]
     double2* B = A + kTileF * Nwex;                  // [kTileF t2][Nwex]
     const double w1 = CH == G4_PH_MAGNETIC ? -1.0 : 1.0;  // weight of spin -1 in a, b
-    // G(K2, K1) of the tile (the transverse channel pairs the opposite spin)
-    for (int t = threadIdx.x; t < 2 * kTileF * kTileF; t += blockDim.x) {
-        const int sp = t / (kTileF * kTileF), r = t % (kTileF * kTileF);
-        const int a2 = r / kTileF, a1 = r % kTileF;
-        const int m1 = n1_0 + a1, m2 = n2_0 + a2;
-        const int gs = CH == G4_PH_TRANSVERSE ? 1 - sp : sp;
-        X1[(sp * kTileF + a2) * (kTileF + 1) + a1] =
-            (m1 < Nw2 && m2 < Nw2) ? G[gs * NN + (size_t)(k2 * Nw2 + m2) * N + k1 * Nw2 + m1]
-                                   : make_double2(0.0, 0.0);
-    }
     for (int q = 0; q < d.Nkex; ++q) {
         const int k1q = kadd[k1 * d.Nc + q], k2q = kadd[k2 * d.Nc + q];
-        __syncthreads();  // the previous q's tiles are no longer read
-        for (int t = threadIdx.x; t < 2 * WX * WX; t += blockDim.x) {
-            const int sp = t / (WX * WX), r = t % (WX * WX);
-            const int i = r / WX, j = r % WX;
-            const int f1 = n1_0 + i + d.m0, f2 = n2_0 + j + d.m0;  // frequencies n + m
-            X2[(sp * WX + i) * (WX + 1) + j] =
-                (f1 < Nw2 && f2 < Nw2) ? G[sp * NN + (size_t)(k1q * Nw2 + f1) * N + k2q * Nw2 + f2]
-                                       : make_double2(0.0, 0.0);
-        }
-        if (CH != G4_PH_TRANSVERSE) {
-            for (int t = threadIdx.x; t < 2 * kTileF * Nwex; t += blockDim.x) {
-                const int side = t / (kTileF * Nwex), r = t % (kTileF * Nwex);
-                const int u = r / Nwex, m = r % Nwex;
-                const int mg = d.m0 + m;
+        double2 sum[WXM];
+#pragma unroll
+        for (int m = 0; m < WXM; ++m) sum[m] = make_double2(0.0, 0.0);
+        for (int r = 0; r < staged; ++r) {
+            const double2* G = Gb + (size_t)(2 * r) * NN;
+            const double sign = signs.s[r];
+            __syncthreads();  // the previous tiles are no longer read
+            // G(K2, K1) of the tile (the transverse channel pairs the opposite spin)
+            for (int t = threadIdx.x; t < 2 * kTileF * kTileF; t += blockDim.x) {
+                const int sp = t / (kTileF * kTileF), u = t % (kTileF * kTileF);
+                const int a2 = u / kTileF, a1 = u % kTileF;
+                const int m1 = n1_0 + a1, m2 = n2_0 + a2;
+                const int gs = CH == G4_PH_TRANSVERSE ? 1 - sp : sp;
                 double2 v = make_double2(0.0, 0.0);
-                if (side == 0) {
-                    // a(n1, m) = sum_s w_s G_s((k1 (+) q, n1 + m), (k1, n1))
-                    const int nn = n1_0 + u;
-                    if (nn < Nw2 && nn + mg < Nw2) {
-                        const size_t i0 = (size_t)(k1q * Nw2 + nn + mg) * N + k1 * Nw2 + nn;
-                        const double2 g0 = G[i0], g1 = G[NN + i0];
-                        v = make_double2(g0.x + w1 * g1.x, g0.y + w1 * g1.y);
-                    }
-                    A[u * Nwex + m] = v;
-                } else {
+                if (m1 < Nw2 && m2 < Nw2) v = G[gs * NN + (size_t)(k2 * Nw2 + m2) * N + k1 * Nw2 + m1];
+                X1[(sp * kTileF + a2) * (kTileF + 1) + a1] = make_double2(-sign * v.x, -sign * v.y);
+            }
+            for (int t = threadIdx.x; t < 2 * WX * WX; t += blockDim.x) {
+                const int sp = t / (WX * WX), u = t % (WX * WX);
+                const int i = u / WX, j = u % WX;
+                const int f1 = n1_0 + i + d.m0, f2 = n2_0 + j + d.m0;  // frequencies n + m
+                X2[(sp * WX + i) * (WX + 1) + j] =
+                    (f1 < Nw2 && f2 < Nw2) ? G[sp * NN + (size_t)(k1q * Nw2 + f1) * N + k2q * Nw2 + f2]
+                                           : make_double2(0.0, 0.0);
+            }
+            if (CH != G4_PH_TRANSVERSE) {
+                for (int t = threadIdx.x; t < 2 * kTileF * Nwex; t += blockDim.x) {
+                    const int side = t / (kTileF * Nwex), w = t % (kTileF * Nwex);
+                    const int u = w / Nwex, m = w % Nwex;
+                    const int mg = d.m0 + m;
+                    double2 v = make_double2(0.0, 0.0);
+                    // a(n1, m) = sum_s w_s G_s((k1 (+) q, n1 + m), (k1, n1)),
                     // b(n2, m) = sum_s w_s G_s((k2, n2), (k2 (+) q, n2 + m))
-                    const int nn = n2_0 + u;
+                    const int nn = (side ? n2_0 : n1_0) + u;
                     if (nn < Nw2 && nn + mg < Nw2) {
-                        const size_t i0 = (size_t)(k2 * Nw2 + nn) * N + k2q * Nw2 + nn + mg;
+                        const size_t i0 = side ? (size_t)(k2 * Nw2 + nn) * N + k2q * Nw2 + nn + mg
+                                               : (size_t)(k1q * Nw2 + nn + mg) * N + k1 * Nw2 + nn;
                         const double2 g0 = G[i0], g1 = G[NN + i0];
-                        v = make_double2(g0.x + w1 * g1.x, g0.y + w1 * g1.y);
+                        const double f = side ? 1.0 : sign;
+                        v = make_double2(f * (g0.x + w1 * g1.x), f * (g0.y + w1 * g1.y));
                     }
-                    B[u * Nwex + m] = v;
+                    (side ? B : A)[w] = v;
                 }
             }
+            __syncthreads();
+#pragma unroll
+            for (int m = 0; m < WXM; ++m) {
+                if (m >= Nwex) break;
+                if (CH != G4_PH_TRANSVERSE) cfma(sum[m], A[t1 * Nwex + m], B[t2 * Nwex + m]);
+#pragma unroll
+                for (int sp = 0; sp < 2; ++sp)
+                    cfma(sum[m], X1[(sp * kTileF + t2) * (kTileF + 1) + t1],
+                         X2[(sp * WX + t1 + m) * (WX + 1) + t2 + m]);
+            }
         }
-        __syncthreads();
         if (!live) continue;
         double2* row = acc + ((size_t)(k1 * Nw2 + n1) * N + k2 * Nw2 + n2) * d.NQ + (size_t)q * Nwex;
-        for (int m = 0; m < Nwex; ++m) {
-            if (n1 + d.m0 + m >= Nw2 || n2 + d.m0 + m >= Nw2) continue;  // structurally zero
-            double2 term = make_double2(0.0, 0.0);
-            if (CH != G4_PH_TRANSVERSE) term = cmul(A[t1 * Nwex + m], B[t2 * Nwex + m]);
 #pragma unroll
-            for (int sp = 0; sp < 2; ++sp) {
-                const double2 e = cmul(X1[(sp * kTileF + t2) * (kTileF + 1) + t1],
-                                       X2[(sp * WX + t1 + m) * (WX + 1) + t2 + m]);
-                term.x -= e.x;
-                term.y -= e.y;
-            }
+        for (int m = 0; m < WXM; ++m) {
+            if (m >= Nwex) break;
+            if (n1 + d.m0 + m >= Nw2 || n2 + d.m0 + m >= Nw2) continue;  // structurally zero
             double2 o = row[m];
-            o.x += sign * term.x;
-            o.y += sign * term.y;
+            o.x += sum[m].x;
+            o.y += sum[m].y;
             row[m] = o;
         }
     }
@@ -378,67 +423,73 @@ __global__ void __launch_bounds__(256) k_build_G_diag(const void* __restrict__ M
     }
 }
 
-int grid_for(size_t work, int block) {
-    size_t g = (work + block - 1) / block;
-    if (g > (size_t)152 * 64) g = (size_t)152 * 64;
-    return (int)(g ? g : 1);
-}
+constexpr long long kTiledMinEntries = 1 << 18;
 
 }  // namespace
 
 cudaError_t launch_build_G_fp64(const void* M, bool m64, const double2* G0, double2* G, int N,
-                                cudaStream_t s) {
-    const size_t total = 2 * (size_t)N * N;
-    const int g = grid_for(total, 256);
+                                unsigned* flag, cudaStream_t s) {
+    const int bx = N >= 256 ? 256 : (N + 31) / 32 * 32;
+    const dim3 grid((N + kBuildU * bx - 1) / (kBuildU * bx), std::min(2LL * N, 65535LL));
     if (m64)
-        k_build_G_fp64<true><<<g, 256, 0, s>>>(M, G0, G, N);
+        k_build_G_fp64<true><<<grid, bx, 0, s>>>(M, G0, G, N, flag);
     else
-        k_build_G_fp64<false><<<g, 256, 0, s>>>(M, G0, G, N);
+        k_build_G_fp64<false><<<grid, bx, 0, s>>>(M, G0, G, N, flag);
     return cudaGetLastError();
 }
 
-cudaError_t launch_update_fp64(const double2* G, double sign, double2* acc, const int* kadd,
-                               const int* ksub, const G4Dims& d, cudaStream_t s) {
-    if (d.ch != G4_PP_UPDOWN && d.Nwex <= kTileWex && (long long)d.Nc * d.Nc <= 65535) {
+namespace {
+template <int CH>
+cudaError_t update_fp64(const double2* G, const G4Signs& signs, int staged, double2* acc,
+                        const int* kadd, const int* ksub, const G4Dims& d, const unsigned* only_if,
+                        cudaStream_t s) {
+    // the tiled kernel from 2^18 entries on; below, a launch of it is a chain of
+    // barriers over transfers and measurements in a few blocks
+    if (CH != G4_PP_UPDOWN && d.Nwex <= kTileWex && (long long)d.Nc * d.Nc <= 65535 &&
+        d.E >= kTiledMinEntries) {
         const int nt = (d.Nw2 + kTileF - 1) / kTileF;
         const int WX = kTileF + d.Nwex - 1;
         const size_t smem = (2 * (size_t)WX * (WX + 1) + 2 * kTileF * (kTileF + 1) +
                              2 * (size_t)kTileF * d.Nwex) * sizeof(double2);
         const dim3 grid(nt * nt, d.Nc * d.Nc);
-        cudaError_t e;
-        switch (d.ch) {
-            case G4_PH_DENSITY:
-                if ((e = raise_smem_limit(k_update_fp64_tiled<G4_PH_DENSITY>)) != cudaSuccess) return e;
-                k_update_fp64_tiled<G4_PH_DENSITY><<<grid, kTileF * kTileF, smem, s>>>(G, sign, acc, kadd, d);
-                break;
-            case G4_PH_TRANSVERSE:
-                if ((e = raise_smem_limit(k_update_fp64_tiled<G4_PH_TRANSVERSE>)) != cudaSuccess) return e;
-                k_update_fp64_tiled<G4_PH_TRANSVERSE><<<grid, kTileF * kTileF, smem, s>>>(G, sign, acc, kadd, d);
-                break;
-            default:
-                if ((e = raise_smem_limit(k_update_fp64_tiled<G4_PH_MAGNETIC>)) != cudaSuccess) return e;
-                k_update_fp64_tiled<G4_PH_MAGNETIC><<<grid, kTileF * kTileF, smem, s>>>(G, sign, acc, kadd, d);
+        auto* k = d.Nwex <= 4 ? k_update_fp64_tiled<CH, 4>
+                              : d.Nwex <= 8 ? k_update_fp64_tiled<CH, 8> : k_update_fp64_tiled<CH, kTileWex>;
+        if (smem > 48 * 1024) {
+            cudaError_t e = raise_smem_limit(k);
+            if (e != cudaSuccess) return e;
         }
+        k<<<grid, kTileF * kTileF, smem, s>>>(G, signs, staged, acc, kadd, d, only_if);
         return cudaGetLastError();
     }
     const int per = d.N * d.NQ;
-    int gx = (per + 255) / 256;
-    if (gx > 64) gx = 64;
-    dim3 grid(gx, d.N);
+    auto run = [&](auto rs) {
+        constexpr int RS = decltype(rs)::value;
+        const long long threads = (long long)per * RS;
+        const int bx = threads < 256 ? (int)(threads + 31) / 32 * 32 : 256;
+        const int gx = (int)std::min<long long>((threads + bx - 1) / bx, 64);
+        k_update_fp64<CH, RS><<<dim3(gx, d.N), bx, 0, s>>>(G, signs, staged, acc, kadd, ksub, d, only_if);
+    };
+    // a lane per entry once that fills the GPU a few times over
+    if (d.E >= (1 << 18) || staged < 4) run(std::integral_constant<int, 1>());
+    else if (d.E >= (1 << 15) || staged < 16) run(std::integral_constant<int, 4>());
+    else run(std::integral_constant<int, 16>());
+    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_update_fp64(const double2* G, const G4Signs& signs, int staged, double2* acc,
+                               const int* kadd, const int* ksub, const G4Dims& d,
+                               const unsigned* only_if, cudaStream_t s) {
     switch (d.ch) {
         case G4_PP_UPDOWN:
-            k_update_fp64<G4_PP_UPDOWN><<<grid, 256, 0, s>>>(G, sign, acc, kadd, ksub, d);
-            break;
+            return update_fp64<G4_PP_UPDOWN>(G, signs, staged, acc, kadd, ksub, d, only_if, s);
         case G4_PH_DENSITY:
-            k_update_fp64<G4_PH_DENSITY><<<grid, 256, 0, s>>>(G, sign, acc, kadd, ksub, d);
-            break;
+            return update_fp64<G4_PH_DENSITY>(G, signs, staged, acc, kadd, ksub, d, only_if, s);
         case G4_PH_TRANSVERSE:
-            k_update_fp64<G4_PH_TRANSVERSE><<<grid, 256, 0, s>>>(G, sign, acc, kadd, ksub, d);
-            break;
+            return update_fp64<G4_PH_TRANSVERSE>(G, signs, staged, acc, kadd, ksub, d, only_if, s);
         default:
-            k_update_fp64<G4_PH_MAGNETIC><<<grid, 256, 0, s>>>(G, sign, acc, kadd, ksub, d);
+            return update_fp64<G4_PH_MAGNETIC>(G, signs, staged, acc, kadd, ksub, d, only_if, s);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_finalize(const double2* acc, bool pair, double inv_s, double2* out,

@@ -61,6 +61,7 @@
 
 #include <type_traits>
 
+#include "g4_diag.cuh"
 #include "g4_gtilde.cuh"
 #include "g4_internal.h"
 #include "g4_ptx.cuh"
@@ -245,15 +246,6 @@ struct PackM {
     // stages, D = 0 positions, slot sign factors, full and empty mbarriers, flag
     static constexpr int SMEM = NST * STAGE + MAXNC * 4 + kMaxBatch * 8 + 2 * NST * 8 + 16;
 };
-
-// Position of diagonal (dk, dn) in the exchange's diagonal list: (D, -D) pairs
-// in the order dn = 0, 1, ... with dk inner, dn = 0 listed once per pair
-// (pos0, a table of Nc entries); mk = (-)dk.
-__device__ __forceinline__ int diag_pos(int dk, int dn, int mk, int Nc, const int* pos0) {
-    if (dn > 0) return Nc + (dn - 1) * 2 * Nc + 2 * dk;
-    if (dn < 0) return Nc + (-dn - 1) * 2 * Nc + 2 * mk + 1;
-    return pos0[dk];
-}
 
 __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
     asm volatile(
@@ -1414,31 +1406,7 @@ g4_status xtc_prepare(g4_ctx* h) {
         return g4_fail(h, G4_ERR_INVALID, "padded batch is not a whole number of operand chunks");
     X->aoff = (d.ch == G4_PH_TRANSVERSE || d.ch == G4_PP_UPDOWN) ? X->Jh / chunk_of(X->f16) : 0;
 
-    // diagonals in pairs (D, -D), so that a diagonal read as A is read as B soon after
-    std::vector<int> ksub((size_t)d.Nc * d.Nc);
-    for (int a = 0; a < d.Nc; ++a)
-        for (int b = 0; b < d.Nc; ++b) {
-            const int ax = a % d.Lx, ay = a / d.Lx, bx = b % d.Lx, by = b / d.Lx;
-            ksub[a * d.Nc + b] = (ax - bx + d.Lx) % d.Lx + d.Lx * ((ay - by + d.Ly) % d.Ly);
-        }
-    for (int dn = 0; dn < d.Nw2; ++dn)
-        for (int dk = 0; dk < d.Nc; ++dk) {
-            const int mk = ksub[0 * d.Nc + dk];
-            if (dn == 0) {
-                if (mk < dk) continue;
-                X->dl.push_back(make_int2(dk, 0));
-                if (mk != dk) {
-                    X->dl.push_back(make_int2(mk, 0));
-                    X->itemlen.push_back(2);
-                } else {
-                    X->itemlen.push_back(1);
-                }
-            } else {
-                X->dl.push_back(make_int2(dk, dn));
-                X->dl.push_back(make_int2(mk, -dn));
-                X->itemlen.push_back(2);
-            }
-        }
+    diag_list(d, X->dl, X->itemlen);
     // one diagonal of the group, both planes
     const size_t per_slot = (size_t)d.Nc * d.Nw2 * 2 * X->J * (X->f16 ? 2 : 4) * 2;
     size_t budget = h->deferred ? kXBudgetDeferred : kXBudget;

@@ -36,6 +36,12 @@ struct G4SlotTable {
     G4Slot s[kMaxBatch];
 };
 
+// Signs of the measurements an FP64 handle has staged (at most 64), passed to
+// the kernels by value.
+struct G4Signs {
+    double s[64];
+};
+
 // Channels with a direct (outer-product) term: the magnetic and density forms.
 inline bool has_direct(int ch) { return ch == G4_PH_MAGNETIC || ch == G4_PH_DENSITY; }
 
@@ -98,8 +104,11 @@ struct g4_ctx {
     unsigned* gredo = nullptr;       // deferred staging: the pack has to run again
     unsigned* hstatus = nullptr;     // pinned host mirror
 
-    // FP64 plain path
+    // FP64 path
     double2* Gfull = nullptr;        // [batch][2][N][N]
+    void* f64tc = nullptr;           // batch update on tensor cores (g4_fp64_tc.cu), or null;
+                                     // *gmax is then the batch's flag: a G entry that only
+                                     // the plain kernels take
 
     // mixed path
     float2* Gd = nullptr;            // [batch*2][Nc dk][ndn][Nc k][Nw2 n] complex64,
@@ -152,10 +161,24 @@ g4_status g4_cuda_fail(g4_ctx* h, cudaError_t e, const char* what);
 g4_status g4_dalloc_bytes(g4_ctx* h, void** p, size_t bytes);
 
 // kernels (launch wrappers), each returns cudaGetLastError()
+// flag (may be null) is set when a component of G is not finite or outside
+// 2^+-kF64tcExp (zero is inside)
+constexpr int kF64tcExp = 380;
 cudaError_t launch_build_G_fp64(const void* M, bool m64, const double2* G0, double2* G,
-                                int N, cudaStream_t s);
-cudaError_t launch_update_fp64(const double2* G, double sign, double2* acc, const int* kadd,
-                               const int* ksub, const G4Dims& d, cudaStream_t s);
+                                int N, unsigned* flag, cudaStream_t s);
+// the staged measurements' plain FP64 update; with only_if given the launch
+// does nothing unless *only_if is set
+cudaError_t launch_update_fp64(const double2* G, const G4Signs& signs, int staged, double2* acc,
+                               const int* kadd, const int* ksub, const G4Dims& d,
+                               const unsigned* only_if, cudaStream_t s);
+
+// FP64 path, a batch's update on tensor cores (g4_fp64_tc.cu): prepare leaves
+// h->f64tc null where the path does not apply (or its memory is not there)
+constexpr double kF64tcMinUpdates = 4e6;
+void f64tc_prepare(g4_ctx* h);
+bool f64tc_wanted(const g4_ctx* h, int staged);
+g4_status f64tc_run(g4_ctx* h, int staged);
+void f64tc_release(g4_ctx* h);
 // out = acc / S in the exported layout, for the n2 planes [n2_0, n2_0 + n2_cnt):
 // plane m of the block is written at out + m * out_plane (E / Nwex for the
 // whole array with n2_0 = 0, n2_cnt = 2Nw)

@@ -146,6 +146,15 @@ __device__ __forceinline__ int f16_shift(uint32_t maxbits) {
 // 2^e for e in [-126, 127], exactly.
 __device__ __forceinline__ float pow2f(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
 
+// One lane of the (whole) warp, the same one every time.  A warp that issues
+// MMAs runs its loop with all lanes, so that descriptors and addresses are
+// warp-uniform, and enters `if (elect_one())` for the MMAs alone.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
     asm volatile(
         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
