@@ -15,6 +15,7 @@
 // reads, so nothing needs clearing between calls.
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "g4_internal.h"
@@ -61,52 +62,96 @@ __global__ void k_na_build(const double2* __restrict__ M, const double2* __restr
     }
 }
 
-// acc[m][n2][n1][q][k2][k1] += sign * (a b - exchange), one thread per entry.
-__global__ void k_na_update(const double2* __restrict__ G, double sign, double2* __restrict__ acc,
-                            int Nc, int Lx, int Nw2, int Nwex, int Nkex) {
-    const int N = Nc * Nw2, Ly = Nc / Lx;
+// acc[m][n2][n1][q][k2][k1] += sign * (a b - exchange).  A block takes gp
+// consecutive (n1, q) of one n2 (blockIdx.y), its threads the gp Nc^2 pairs
+// (k2, k1) of each, and walks the transfers m in steps of kNaM: a (with the
+// sign) and b of the step are formed once into shared memory, G(K2, K1) is read
+// once per entry, the kNaM accumulator entries and G(K1+Q, K2+Q) are read
+// together.  Bound by the FP64 pipe (two lanes per clock and SM): fourteen
+// operations per entry, and no index division or weighted sum per entry (one
+// thread per entry with both took 211 us for N = 256 and 64 transfers; this
+// 110).  The contribution is summed before it meets the accumulator: with the
+// accumulator inside the chain of fused multiply-adds, two operations fewer
+// (95 us), the error against 64 bits grew by half.
+constexpr int kNaM = 4;
+constexpr int kNaThreads = 256;
+
+__device__ __forceinline__ void na_cfma(double2& t, double2 a, double2 b) {
+    t.x = fma(a.x, b.x, t.x);
+    t.y = fma(a.x, b.y, t.y);
+    t.x = fma(-a.y, b.y, t.x);
+    t.y = fma(a.y, b.x, t.y);
+}
+
+__global__ void __launch_bounds__(kNaThreads) k_na_update(const double2* __restrict__ G, double sign,
+                                                          double2* __restrict__ acc, int Nc, int Lx,
+                                                          int Nw2, int Nwex, int Nkex, int gp) {
+    __shared__ double2 sa[kNaM * kNaThreads], sb[kNaM * kNaThreads];   // [m][group][k]
+    const int N = Nc * Nw2, Ly = Nc / Lx, N2 = Nc * Nc;
     const size_t NN = (size_t)N * N;
-    const long long E = (long long)N * N * Nkex * Nwex;
-    for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < E;
-         o += (long long)gridDim.x * blockDim.x) {
-        long long t = o;
-        const int k1 = (int)(t % Nc); t /= Nc;
-        const int k2 = (int)(t % Nc); t /= Nc;
-        const int q = (int)(t % Nkex); t /= Nkex;
-        const int n1 = (int)(t % Nw2); t /= Nw2;
-        const int n2 = (int)(t % Nw2);
-        const int m = (int)(t / Nw2);
-        const int qx = q % Lx, qy = q / Lx;
-        const int k1q = (k1 % Lx + qx) % Lx + Lx * ((k1 / Lx + qy) % Ly);
-        const int k2q = (k2 % Lx + qx) % Lx + Lx * ((k2 / Lx + qy) % Ly);
-        const int K1 = k1 * Nw2 + n1, K2 = k2 * Nw2 + n2;
-        const bool v1 = n1 + m < Nw2, v2 = n2 + m < Nw2;
-        const int K1Q = k1q * Nw2 + n1 + m, K2Q = k2q * Nw2 + n2 + m;
-        double2 a = make_double2(0, 0), b = make_double2(0, 0), ex = make_double2(0, 0);
-        for (int sp = 0; sp < 2; ++sp) {
-            const double2* g = G + sp * NN;
-            const double sg = sp ? -1.0 : 1.0;
-            if (v1) {
-                const double2 u = g[(size_t)K1Q * N + K1];
-                a.x += sg * u.x;
-                a.y += sg * u.y;
-            }
-            if (v2) {
-                const double2 u = g[(size_t)K2 * N + K2Q];
-                b.x += sg * u.x;
-                b.y += sg * u.y;
-            }
-            if (v1 && v2) {
-                const double2 u = na_cmul(g[(size_t)K2 * N + K1], g[(size_t)K1Q * N + K2Q]);
-                ex.x += u.x;
-                ex.y += u.y;
+    const int n2 = blockIdx.y, g0 = blockIdx.x * gp, ng = min(gp, Nw2 * Nkex - g0);
+    const size_t plane = (size_t)Nw2 * Nkex * N2;   // entries of one (m, n2)
+    auto add = [&](int k, int q) {
+        int x = k % Lx + q % Lx, y = k / Lx + q / Lx;
+        x -= x >= Lx ? Lx : 0;
+        y -= y >= Ly ? Ly : 0;
+        return x + Lx * y;
+    };
+    for (int m0 = 0; m0 < Nwex; m0 += kNaM) {
+        __syncthreads();
+        for (int t = threadIdx.x; t < ng * Nc; t += blockDim.x) {
+            const int g = t / Nc, k = t - g * Nc;
+            const int n1 = (g0 + g) / Nkex, q = (g0 + g) - n1 * Nkex;
+            const int kq = add(k, q);
+#pragma unroll
+            for (int u = 0; u < kNaM; ++u) {
+                const int m = m0 + u;
+                double2 a = make_double2(0.0, 0.0), b = a;
+                if (m < Nwex && n1 + m < Nw2) {
+                    const size_t e = (size_t)(kq * Nw2 + n1 + m) * N + k * Nw2 + n1;
+                    const double2 x = G[e], y = G[NN + e];
+                    a = make_double2(sign * (x.x - y.x), sign * (x.y - y.y));
+                }
+                if (m < Nwex && n2 + m < Nw2) {
+                    const size_t e = (size_t)(k * Nw2 + n2) * N + kq * Nw2 + n2 + m;
+                    const double2 x = G[e], y = G[NN + e];
+                    b = make_double2(x.x - y.x, x.y - y.y);
+                }
+                sa[u * kNaThreads + t] = a;
+                sb[u * kNaThreads + t] = b;
             }
         }
-        const double2 ab = na_cmul(a, b);
-        double2 r = acc[o];
-        r.x += sign * (ab.x - ex.x);
-        r.y += sign * (ab.y - ex.y);
-        acc[o] = r;
+        __syncthreads();
+        for (int t = threadIdx.x; t < ng * N2; t += blockDim.x) {
+            const int g = t / N2, r = t - g * N2, k2 = r / Nc, k1 = r - k2 * Nc;
+            const int n1 = (g0 + g) / Nkex, q = (g0 + g) - n1 * Nkex;
+            const int lim = min(Nwex, Nw2 - max(n1, n2)) - m0;   // transfers on the grid
+            if (lim <= 0) continue;
+            const size_t e1 = (size_t)(k2 * Nw2 + n2) * N + k1 * Nw2 + n1;
+            const size_t e2 = (size_t)(add(k1, q) * Nw2 + n1 + m0) * N + add(k2, q) * Nw2 + n2 + m0;
+            double2* o = acc + (size_t)m0 * Nw2 * plane + (size_t)n2 * plane + (size_t)g0 * N2 + t;
+            double2 x1[2], x2[kNaM][2], s[kNaM];
+#pragma unroll
+            for (int sp = 0; sp < 2; ++sp) {
+                x1[sp] = G[sp * NN + e1];
+                x1[sp] = make_double2(-sign * x1[sp].x, -sign * x1[sp].y);
+            }
+#pragma unroll
+            for (int u = 0; u < kNaM; ++u)
+                if (u < lim) {
+                    s[u] = o[(size_t)u * Nw2 * plane];
+#pragma unroll
+                    for (int sp = 0; sp < 2; ++sp) x2[u][sp] = G[sp * NN + e2 + (size_t)u * (N + 1)];
+                }
+#pragma unroll
+            for (int u = 0; u < kNaM; ++u)
+                if (u < lim) {
+                    double2 v = na_cmul(x1[0], x2[u][0]);
+                    na_cfma(v, x1[1], x2[u][1]);
+                    na_cfma(v, sa[u * kNaThreads + g * Nc + k1], sb[u * kNaThreads + g * Nc + k2]);
+                    o[(size_t)u * Nw2 * plane] = make_double2(s[u].x + v.x, s[u].y + v.y);
+                }
+        }
     }
 }
 
@@ -194,10 +239,10 @@ extern "C" g4_status g4_update_noalloc(int Nc, int lx, int Nw, int Nwex, int Nke
     k_na_build<<<blocks, 256, 0, s>>>((const double2*)M, (const double2*)G0, G, (int)N);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(G4_ERR_CUDA, std::string("build launch: ") + cudaGetErrorString(e));
-    const long long E = N * N * Nkex * Nwex;
-    long long ub = (E + 255) / 256;
-    if (ub > 152 * 32) ub = 152 * 32;
-    k_na_update<<<(int)ub, 256, 0, s>>>(G, sign, (double2*)acc, Nc, Lx, 2 * Nw, Nwex, Nkex);
+    // (n1, q) groups per block: as many whole Nc x Nc planes as its threads hold
+    const int gp = std::max(1, kNaThreads / (Nc * Nc)), groups = 2 * Nw * Nkex;
+    k_na_update<<<dim3((groups + gp - 1) / gp, 2 * Nw), kNaThreads, 0, s>>>(G, sign, (double2*)acc, Nc, Lx, 2 * Nw,
+                                                                            Nwex, Nkex, gp);
     e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(G4_ERR_CUDA, std::string("update launch: ") + cudaGetErrorString(e));
     return G4_OK;
