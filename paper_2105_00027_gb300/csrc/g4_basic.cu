@@ -342,85 +342,102 @@ __global__ void k_finalize_gather(const double2* __restrict__ acc, double inv_s,
     }
 }
 
-// Mixed path G build.  One block owns the (row momentum kr, column momentum kc)
-// frequency block of one spin: it forms G in FP32, scales it by sqrt(s_r)
+// Mixed path G build.  One block owns kDiagCols columns c = (kc, j) of one row
+// momentum kr and spin: it forms G in FP32, scales it by sqrt(s_r)
 // (i sqrt(|s_r|) for a negative sign, so that the product of two entries of
-// the same measurement carries s_r), rounds to complex64 into a padded shared
-// tile, then writes every frequency-difference diagonal of the block into its
-// Nw2-long row (the positions where the row index leaves the grid stay zero):
+// the same measurement carries s_r) and writes every frequency-difference
+// diagonal's complex64 run over its columns (the positions where the row index
+// leaves the grid stay zero):
 //   Gd[j][dk][dn + Nw2-1][kc][n] = sqrt(s_r) G((kr, n+dn), (kc, n)),  kr = kc (+) dk.
-// WRITE = false is the same pass without the tile and the writes: only the
-// largest component joins *gmax (the deferred staging's per-measurement pass).
-template <bool M64, bool WRITE>
+//
+// Bound by HBM (M read once, G~ written once).  The Nw2 rows of M go to shared
+// memory by asynchronous copies, all in flight at once without holding
+// registers, and are read back along the diagonals: a lane's row stride is a
+// multiple of 128 bytes and lanes are consecutive columns, so every access is
+// free of bank conflicts.  Step t takes row (n + t) mod Nw2, whose diagonal is
+// dn = t or t - Nw2: all lanes write in every step, where walking the 2Nw2 - 1
+// diagonals in turn left half of them out.  Columns run over momenta, so small
+// frequency counts fill their warps too.  One maximum per block goes to *gmax.
+// Measured back to back (bytes M + G~), before -> after, complex128 M:
+// N = 32: 4.17 -> 2.15 us; N = 1024 (4x4, 64 frequencies):
+// 18.9 -> 14.4 us (3.5 TB/s); N = 2304: 61.7 -> 50.6 us (5.0 TB/s); complex64,
+// N = 750 (50 frequencies): 12.3 -> 7.9 us.  Of that the programmatic launch is
+// 2 us; 16 columns or 128 threads per block measured within 5% either way, 512
+// threads 10% slower at N = 2304.
+constexpr int kDiagCols = 32;
+
+template <typename MV>
+__device__ __forceinline__ void cp_async_entry(void* dst, const MV* src) {
+    if constexpr (sizeof(MV) == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(g4ptx::smem_u32(dst)), "l"(src) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(g4ptx::smem_u32(dst)), "l"(src) : "memory");
+}
+
+__device__ __forceinline__ float2 narrow(float2 z) { return z; }
+__device__ __forceinline__ float2 narrow(double2 z) {
+    return make_float2(g4ptx::f64_to_f32(z.x), g4ptx::f64_to_f32(z.y));
+}
+
+template <bool M64>
 __global__ void __launch_bounds__(256) k_build_G_diag(const void* __restrict__ M,
-                                                      const double2* __restrict__ G0, double sign,
-                                                      float2* __restrict__ Gd,
+                                                      const double2* __restrict__ G0,
+                                                      g4gt::SignFactor sf, float2* __restrict__ Gd,
                                                       const int* __restrict__ ksub, G4Dims d,
                                                       unsigned* __restrict__ gmax) {
-    extern __shared__ float2 tile[];  // [Nw2][Nw2+2] (WRITE), then G0 of the block's rows [Nw2]
-    const int kc = blockIdx.x, kr = blockIdx.y, sp = blockIdx.z;
-    const int Nw2 = d.Nw2, N = d.N, ld = Nw2 + 2;
-    const size_t NN = (size_t)N * N;
-    float2* g0row = tile + (WRITE ? Nw2 * ld : 0);
-    // complex64 storage: form G in FP32 (three roundings, below the storage rounding scale)
-    const g4gt::SignFactor sf = g4gt::sign_factor(sign);
-    for (int i = threadIdx.x; i < Nw2; i += blockDim.x) {
-        const double2 g = G0[sp * N + kr * Nw2 + i];
-        g0row[i] = make_float2((float)g.x, (float)g.y);
-    }
-    __syncthreads();
-    // Thread layout: a fixed column j = tid % Nw2 and rows i = tid / Nw2 + RPB*k
-    // (RPB rows per sweep), so no per-element division; U independent loads of
-    // M per thread are in flight before any is used (eight 8-byte loads of a
-    // complex64 M or four 16-byte loads of a complex128 one; sixteen with a
-    // register cap for three blocks per SM measured 12% slower).
-    const int RPB = blockDim.x / Nw2 > 0 ? blockDim.x / Nw2 : 1;
-    const int j = threadIdx.x % Nw2, i0 = threadIdx.x / Nw2;
-    const bool lane_ok = i0 < RPB;  // threads beyond RPB*Nw2 (Nw2 not dividing the block) idle
-    const double2 gj64 = G0[sp * N + kc * Nw2 + j];
-    const float2 gj = make_float2((float)gj64.x, (float)gj64.y);
-    const size_t mbase = sp * NN + (size_t)(kr * Nw2) * N + kc * Nw2 + j;
-    constexpr int U = M64 ? 8 : 4;
-    float vmax = 0.f;
     // M entries as loaded: complex64 stays complex64, complex128 is narrowed below
     using MV = typename std::conditional<M64, float2, double2>::type;
-    if (lane_ok) {
-        for (int ib = i0; ib < Nw2; ib += U * RPB) {
-            MV mv[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = ib + u * RPB;
-                if (i < Nw2) mv[u] = reinterpret_cast<const MV*>(M)[mbase + (size_t)i * N];
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int i = ib + u * RPB;
-                if (i >= Nw2) break;
-                const float2 v = g4gt::g_tilde(g0row[i], g4gt::to_c64(mv[u]), gj, kr == kc && i == j, sf);
-                if constexpr (WRITE) tile[i * ld + j] = v;
-                vmax = fmaxf(vmax, fmaxf(fabsf(v.x), fabsf(v.y)));
-            }
+    extern __shared__ __align__(16) unsigned char smem_diag[];
+    __shared__ unsigned bmax;
+    const int Nw2 = d.Nw2, N = d.N;
+    MV* rows = reinterpret_cast<MV*>(smem_diag);                             // [Nw2][kDiagCols]
+    float2* g0row = reinterpret_cast<float2*>(rows + (size_t)Nw2 * kDiagCols);   // [Nw2]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const int c = blockIdx.x * kDiagCols + lane, kr = blockIdx.y, sp = blockIdx.z;
+    const bool ok = c < N;
+    // M and G0 may come from the kernel before: nothing is read until it is done
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const MV* src = reinterpret_cast<const MV*>(M) + ((size_t)sp * N + (size_t)kr * Nw2) * N + c;
+    if (ok)
+        for (int i = warp; i < Nw2; i += nwarp)
+            cp_async_entry(&rows[i * kDiagCols + lane], src + (size_t)i * N);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    // complex64 storage: form G in FP32 (three roundings, below the storage rounding scale)
+    for (int i = threadIdx.x; i < Nw2; i += blockDim.x) {
+        const double2 g = G0[sp * N + kr * Nw2 + i];
+        g0row[i] = narrow(g);
+    }
+    if (threadIdx.x == 0) bmax = 0u;
+    const int kc = ok ? c / Nw2 : 0, n = ok ? c - kc * Nw2 : 0;
+    float2 gj = make_float2(0.f, 0.f);
+    if (ok) {
+        const double2 g = G0[sp * N + c];
+        gj = narrow(g);
+    }
+    const size_t plane = (size_t)d.Nc * Nw2;
+    float2* out = Gd + ((size_t)sp * d.Nc + ksub[kr * d.Nc + kc]) * d.ndn * plane +
+                  (size_t)(Nw2 - 1) * plane + c;   // the diagonal dn = 0
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    float vmax = 0.f;
+    if (ok) {
+#pragma unroll 4
+        for (int t = warp; t < Nw2; t += nwarp) {
+            const bool wrap = n + t >= Nw2;
+            const int dn = wrap ? t - Nw2 : t, i = n + dn;
+            const float2 v = g4gt::g_tilde(g0row[i], narrow(rows[i * kDiagCols + lane]), gj,
+                                           dn == 0 && kr == kc, sf);
+            vmax = fmaxf(vmax, fmaxf(fabsf(v.x), fabsf(v.y)));
+            out[(long long)dn * (long long)plane] = v;
         }
     }
     // the block's largest component joins the batch's maximum (non-negative
     // FP32 values order like their bit patterns)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(gmax, __float_as_uint(vmax));
-    if constexpr (!WRITE) return;
+    const unsigned wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(vmax));
+    if (lane == 0) atomicMax(&bmax, wmax);
     __syncthreads();
-    // Only the in-grid part of each diagonal is written; the out-of-grid part
-    // of every row is zero once and for all (cleared when the handle is made).
-    const int dk = ksub[kr * d.Nc + kc];
-    float2* base = Gd + (((size_t)sp * d.Nc + dk) * d.ndn) * ((size_t)d.Nc * Nw2);
-    if (lane_ok) {
-        const int n = j;
-        for (int dnI = i0; dnI < d.ndn; dnI += RPB) {
-            const int row = n + dnI - (Nw2 - 1);
-            if (row >= 0 && row < Nw2)
-                base[((size_t)dnI * d.Nc + kc) * Nw2 + n] = tile[row * ld + n];
-        }
-    }
+    if (threadIdx.x == 0) atomicMax(gmax, bmax);
 }
 
 constexpr long long kTiledMinEntries = 1 << 18;
@@ -519,14 +536,25 @@ cudaError_t launch_finalize(const double2* acc, bool pair, double inv_s, double2
 cudaError_t launch_build_G_diag(const void* M, bool m64, const double2* G0, double sign,
                                 float2* Gd_slot, const int* ksub, const G4Dims& d,
                                 unsigned* gmax, cudaStream_t s) {
-    // Gd_slot == nullptr: the largest-|G~| pass alone
-    const bool write = Gd_slot != nullptr;
-    const size_t smem = ((write ? (size_t)d.Nw2 * (d.Nw2 + 2) : 0) + d.Nw2) * sizeof(float2);
-    dim3 grid(d.Nc, d.Nc, 2);
-    auto* k = m64 ? (write ? k_build_G_diag<true, true> : k_build_G_diag<true, false>)
-                  : (write ? k_build_G_diag<false, true> : k_build_G_diag<false, false>);
-    cudaError_t e = raise_smem_limit(k);
-    if (e != cudaSuccess) return e;
-    k<<<grid, 256, smem, s>>>(M, G0, sign, Gd_slot, ksub, d, gmax);
-    return cudaGetLastError();
+    const size_t smem = (size_t)d.Nw2 * kDiagCols * (m64 ? sizeof(float2) : sizeof(double2)) +
+                        (size_t)d.Nw2 * sizeof(float2);
+    const dim3 grid((d.N + kDiagCols - 1) / kDiagCols, d.Nc, 2);
+    auto* k = m64 ? k_build_G_diag<true> : k_build_G_diag<false>;
+    if (smem > 48 * 1024) {
+        cudaError_t e = raise_smem_limit(k);
+        if (e != cudaSuccess) return e;
+    }
+    // a run is a chain of these launches: the next one's blocks are set up while
+    // this one finishes, and wait for it (on the device) before their first read
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, M, G0, g4gt::sign_factor(sign), Gd_slot, ksub, d, gmax);
 }
