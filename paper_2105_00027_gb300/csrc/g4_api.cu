@@ -421,6 +421,7 @@ g4_status g4_reset(g4_handle h) {
     G4_CUDA(h, cudaMemsetAsync(h->acc, 0, (size_t)h->d.E * sizeof(double2), h->stream));
     G4_CUDA(h, cudaMemsetAsync(h->dstatus, 0, kStatusWords * sizeof(unsigned), h->stream));
     direct_reset(h);
+    h->scaled = false;
     h->staged = 0;
     h->sign_sum = 0.0;
     h->nmeas = 0;
@@ -761,6 +762,7 @@ g4_status g4_restore(g4_handle h, const char* path) {
     if (st == G4_OK) st = direct_window_max(h, &hd.window_max, false);
     if (st != G4_OK) return st;
     G4_CUDA(h, cudaMemcpy(h->gscale, &hd.gscale, sizeof(unsigned), cudaMemcpyHostToDevice));
+    h->scaled = true;
     h->sign_sum = hd.sign_sum;
     h->nmeas = hd.nmeas;
     h->staged = 0;

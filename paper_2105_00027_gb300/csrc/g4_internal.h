@@ -115,6 +115,7 @@ struct g4_ctx {
                                      // sqrt(s_r) G (so products of two entries carry s_r);
                                      // not allocated on a deferred handle
     bool deferred = false;           // options.deferred: operands formed from M at accumulation
+    bool scaled = false;             // deferred: *gscale may be set (a batch since the reset, or a restore)
     G4SlotTable* slots = nullptr;    // deferred: the staged measurements (host)
     int Bp = 0;                      // padded batch (exchange GEMM K per spin)
     int* pairs = nullptr;            // exchange (k1,q) pairs sorted by p = k1 (+) q
@@ -186,8 +187,7 @@ cudaError_t launch_finalize(const double2* acc, bool pair, double inv_s, double2
                             const G4Dims& d, int n2_0, int n2_cnt, long long out_plane,
                             cudaStream_t s);
 // one measurement's G~ into its batch slot of Gd, its largest component
-// joining *gmax; with Gd_slot == nullptr only the largest component is found
-// (a deferred handle's pass)
+// joining *gmax
 cudaError_t launch_build_G_diag(const void* M, bool m64, const double2* G0, double sign,
                                 float2* Gd_slot, const int* ksub, const G4Dims& d,
                                 unsigned* gmax, cudaStream_t s);
