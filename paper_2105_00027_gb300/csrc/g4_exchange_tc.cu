@@ -1280,6 +1280,8 @@ cudaError_t raise_limits() {
     cudaError_t e;
     if ((e = raise_smem_limit(k_exchange_tc<0, 2, 4, F16>)) != cudaSuccess ||
         (e = raise_smem_limit(k_exchange_tc<1, 2, 4, F16>)) != cudaSuccess ||
+        (e = raise_smem_limit(k_exchange_tc<0, 2, 8, F16>)) != cudaSuccess ||
+        (e = raise_smem_limit(k_exchange_tc<1, 2, 8, F16>)) != cudaSuccess ||
         (e = raise_smem_limit(k_exchange_tc<0, 4, 12, F16>)) != cudaSuccess ||
         (e = raise_smem_limit(k_exchange_tc<1, 4, 12, F16>)) != cudaSuccess ||
         (e = raise_smem_limit(k_exchange_tc<0, 4, 16, F16>)) != cudaSuccess ||
@@ -1300,13 +1302,17 @@ using XKernel = void (*)(const __grid_constant__ CUtensorMap, const __grid_const
 // The kernel variant for a channel geometry (pp: reflected band), window and
 // operand type: the register arrays of the epilogue hold the window W (WM >= W
 // columns per momentum) and the transfers (2 NWH >= Nwex); the narrowest
-// variant that fits does the least work per row.
+// variant that fits does the least work per row, and the epilogue's issue slots
+// are half of what bounds the kernel: 6x6 cluster, 64 frequencies, Nwex = 4 (a
+// window of 5 to 8), two batches of 64: 47.5 ms per run with the <4, 12>
+// variant, 45.0 with <2, 8>; nine problems of 4 to 16 sites, Nwex = 4: 10.3 -> 9.4.
 template <bool F16>
-XKernel pick(bool pp, bool w16, bool wide, bool narrow) {
-    if (narrow) return pp ? k_exchange_tc<1, 2, 4, F16> : k_exchange_tc<0, 2, 4, F16>;
-    if (wide) return pp ? k_exchange_tc<1, 8, 16, F16> : k_exchange_tc<0, 8, 16, F16>;
-    return pp ? (w16 ? k_exchange_tc<1, 4, 16, F16> : k_exchange_tc<1, 4, 12, F16>)
-              : (w16 ? k_exchange_tc<0, 4, 16, F16> : k_exchange_tc<0, 4, 12, F16>);
+XKernel pick(bool pp, int W, int Nwex) {
+    if (Nwex > 8) return pp ? k_exchange_tc<1, 8, 16, F16> : k_exchange_tc<0, 8, 16, F16>;
+    if (Nwex <= 4 && W <= 4) return pp ? k_exchange_tc<1, 2, 4, F16> : k_exchange_tc<0, 2, 4, F16>;
+    if (Nwex <= 4 && W <= 8) return pp ? k_exchange_tc<1, 2, 8, F16> : k_exchange_tc<0, 2, 8, F16>;
+    if (W <= 12) return pp ? k_exchange_tc<1, 4, 12, F16> : k_exchange_tc<0, 4, 12, F16>;
+    return pp ? k_exchange_tc<1, 4, 16, F16> : k_exchange_tc<0, 4, 16, F16>;
 }
 
 }  // namespace
@@ -1673,9 +1679,8 @@ g4_status xtc_run(g4_ctx* h, int staged) {
         prof_end(h, G4_K_PACK_EXCHANGE);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return g4_cuda_fail(h, e, "exchange pack launch");
-        const bool pp = d.ch == G4_PP_UPDOWN, w16 = X->W > 12, wide = d.Nwex > 8;
-        const bool narrow = X->W <= 4 && d.Nwex <= 4;
-        XKernel kern = X->f16 ? pick<true>(pp, w16, wide, narrow) : pick<false>(pp, w16, wide, narrow);
+        const bool pp = d.ch == G4_PP_UPDOWN;
+        XKernel kern = X->f16 ? pick<true>(pp, X->W, d.Nwex) : pick<false>(pp, X->W, d.Nwex);
         // main tiles in runs of two row-frequency blocks of one diagonal, then
         // the split tiles of D = 0 one per block
         for (int part = 0; part < 2; ++part) {
