@@ -147,24 +147,18 @@ g4_status exchange_term(g4_ctx* h) {
 }
 
 // The exchange-type term goes into the accumulator every batch; the direct
-// term's operands join the window, whose GEMM is added when the next batch
-// would not fit (and at g4_finalize).
+// term's operands join the window, whose GEMM is added before a batch that
+// would not fit (the last window's at g4_finalize).  On a deferred handle the
+// exchange pack writes the direct operands at the window's fill, and the window
+// then takes the batch.
 g4_status accumulate_mixed(g4_ctx* h) {
     if (!has_direct(h->d.ch)) return exchange_term(h);
-    bool flush = false;
-    g4_status st;
-    if (h->deferred) {
-        // the exchange pack writes the direct operands at the window's fill;
-        // the window then takes the batch
-        if (direct_fill(h) + h->staged > direct_window(h))
-            return g4_fail(h, G4_ERR_STATE, "direct-term window overflow");
-        if ((st = exchange_term(h)) != G4_OK) return st;
-        if ((st = direct_pack(h, h->staged, &flush)) != G4_OK) return st;
-    } else {
-        if ((st = direct_pack(h, h->staged, &flush)) != G4_OK) return st;
-        if ((st = exchange_term(h)) != G4_OK) return st;
-    }
-    return flush ? direct_flush(h) : G4_OK;
+    g4_status st = G4_OK;
+    if (direct_fill(h) + h->staged > direct_window(h)) st = direct_flush(h);
+    if (st == G4_OK && h->deferred) st = exchange_term(h);
+    if (st == G4_OK) st = direct_pack(h, h->staged);
+    if (st == G4_OK && !h->deferred) st = exchange_term(h);
+    return st;
 }
 
 g4_status do_accumulate(g4_ctx* h) {
@@ -585,7 +579,6 @@ g4_status g4_finalize(g4_handle h, void* out, double* sign_sum) {
     if (h->finalized) return g4_fail(h, G4_ERR_STATE, "g4_finalize called twice");
     g4_status st = do_accumulate(h);
     if (st != G4_OK) return st;
-    if ((st = direct_flush(h)) != G4_OK) return st;
     cudaPointerAttributes attr;
     cudaError_t e = cudaPointerGetAttributes(&attr, out);
     if (e != cudaSuccess) {
@@ -599,9 +592,16 @@ g4_status g4_finalize(g4_handle h, void* out, double* sign_sum) {
     const bool pair = h->opt.accum == G4_ACCUM_F32PAIR;
     const long long plane = d.E / d.Nwex;                     // one m plane of the export
     const long long n2_plane = plane / d.Nw2;                 // one (m, n2) block
-    if (on_device) {
+    // a device output takes the direct term's last window with it; the window
+    // stays (g4_checkpoint then adds it first)
+    const bool with_direct = on_device && direct_finalize_ok(h);
+    if (!with_direct && (st = direct_flush(h)) != G4_OK) return st;
+    if (with_direct) {
+        if ((st = direct_finalize(h, inv, (double2*)out)) != G4_OK) return st;
+    } else if (on_device) {
         prof_begin(h, G4_K_FINALIZE);
-        e = launch_finalize(h->acc, pair, inv, (double2*)out, d, 0, d.Nw2, plane, h->stream);
+        e = launch_finalize(h->acc, pair, inv, (double2*)out, d, 0, d.Nw2, plane, 0, d.Nkex, nullptr,
+                            nullptr, h->stream);
         prof_end(h, G4_K_FINALIZE);
         if (e != cudaSuccess) return g4_cuda_fail(h, e, "finalize launch");
     } else {
@@ -615,8 +615,8 @@ g4_status g4_finalize(g4_handle h, void* out, double* sign_sum) {
         for (int n2 = 0; n2 < d.Nw2 && e == cudaSuccess; n2 += cnt) {
             const int c = std::min(cnt, d.Nw2 - n2);
             prof_begin(h, G4_K_FINALIZE);
-            e = launch_finalize(h->acc, pair, inv, h->hstage, d, n2, c, (long long)c * n2_plane,
-                                h->stream);
+            e = launch_finalize(h->acc, pair, inv, h->hstage, d, n2, c, (long long)c * n2_plane, 0,
+                                d.Nkex, nullptr, nullptr, h->stream);
             prof_end(h, G4_K_FINALIZE);
             const size_t w = (size_t)c * n2_plane * sizeof(double2);
             if (e == cudaSuccess)
@@ -664,6 +664,7 @@ g4_status g4_checkpoint(g4_handle h, const char* path) {
     if (!h || !path) return G4_ERR_INVALID;
     g4_status st = do_accumulate(h);
     if (st != G4_OK) return st;
+    if (h->finalized && (st = direct_flush(h)) != G4_OK) return st;
     if ((st = sync_and_check(h)) != G4_OK) return st;
     const size_t one = (size_t)h->d.E * sizeof(double2);
     const int fill = direct_fill(h);

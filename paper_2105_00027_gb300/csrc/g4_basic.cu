@@ -268,13 +268,6 @@ __global__ void __launch_bounds__(kTileF * kTileF) k_update_fp64_tiled(
     }
 }
 
-// out[m][n2][n1][q][k2][k1] = acc[k1][n1][k2][n2][q][m] * inv_s for n2 in
-// [n2_0, n2_0 + gridDim.y), written at out + m * out_plane + (n2 - n2_0) * (one
-// n2 plane): the whole exported array when out_plane = E / Nwex and n2_0 = 0,
-// or a staging block of a few n2 planes per m.  A block owns one (n1, n2, q)
-// triple and walks k2 in chunks of KC through shared memory: it reads runs of
-// Nwex contiguous entries (all m of one (k1, k2)) and writes runs of KC*Nc
-// contiguous entries (one (m, q) plane).
 // The value of an accumulator entry: complex128, or a pair of complex64 whose
 // sum is the value (compensated FP32 pairs; hi + lo is exact in FP64).
 template <bool PAIR>
@@ -287,58 +280,118 @@ __device__ __forceinline__ double2 acc_value(const double2* acc, size_t i) {
     }
 }
 
-template <bool PAIR>
-__global__ void k_finalize(const double2* __restrict__ acc, double inv_s,
-                           double2* __restrict__ out, G4Dims d, int KC, int n2_0,
-                           long long out_plane) {
-    extern __shared__ double2 tileF[];  // [KC][Nc][Nwex + 1]
-    const int n1 = blockIdx.x, n2l = blockIdx.y, q = blockIdx.z;
-    const int n2 = n2_0 + n2l;
-    const int Nc = d.Nc, Nw2 = d.Nw2, Nwex = d.Nwex, ld = Nwex + 1;
-    for (int k20 = 0; k20 < Nc; k20 += KC) {
-        const int kc = min(KC, Nc - k20);
-        const int cnt = kc * Nc * Nwex;
-        for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-            const int m = t % Nwex;
-            const int r = t / Nwex;
-            const int k1 = r % Nc, k2l = r / Nc;
-            const size_t K1 = (size_t)k1 * Nw2 + n1, K2 = (size_t)(k20 + k2l) * Nw2 + n2;
-            tileF[(k2l * Nc + k1) * ld + m] = acc_value<PAIR>(acc, (K1 * d.N + K2) * d.NQ + (size_t)q * Nwex + m);
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
-            const int r = t % (kc * Nc);       // (k2l, k1), k1 fastest
-            const int m = t / (kc * Nc);
-            const double2 v = tileF[r * ld + m];
-            const size_t o = (size_t)m * out_plane +
-                             (((size_t)n2l * Nw2 + n1) * d.Nkex + q) * Nc * Nc + (size_t)k20 * Nc + r;
-            out[o] = make_double2(v.x * inv_s, v.y * inv_s);
-        }
-        __syncthreads();
-    }
-}
+// out[m][n2][n1][q][k2][k1] = acc[k1][n1][k2][n2][q][m] * inv_s for n2 in
+// [n2_0, n2_0 + n2_cnt) and q in [q0, q0 + nq), written at out + m * out_plane +
+// (n2 - n2_0) * (one n2 plane): the whole exported array when out_plane =
+// E / Nwex and n2_0 = 0, or a staging block of a few n2 planes per m.
+//
+// DIRECT: the direct term's last window is added on the way, acc + scr, in
+// place of a read-modify-write of the accumulator before this pass; scr and
+// scr0 are the group's scratch planes (g4_direct_tc.cu), q0 its first momentum.
+//
+// Bound by HBM, and with DIRECT by the FP64 pipe as much (two additions and two
+// products per entry at two lanes per clock and SM; the sums cannot be formed
+// in fewer without losing bits).  A block owns one n1, kFinN2 consecutive n2
+// and the transfers of TQ momenta (kFinNJ: runs of 128 bytes in the
+// accumulator), and walks the momentum pairs r = (k2, k1) in chunks of RC, a
+// multiple of eight, through kFinBytes of shared memory: out is written in runs
+// of RC entries, whole 128-byte lines.  A thread keeps its transfer and n2 and
+// walks r, so no index is divided inside the loop; kFinU loads of each array
+// are in flight per thread.  Many small blocks keep the FP64 and the memory
+// phases of different blocks side by side.
+// Measured, addition and export, before (read-modify-write by bulk reductions,
+// then export) -> after: 4x4 cluster, 64 frequencies, Nwex = 8: 1.77 -> 1.30 ms;
+// 6x6, 64, 4: 11.4 -> 7.2; 8x8, 32, 4: 15.8 -> 9.9 (4.3 TB/s over acc, scratch
+// and out).  256 threads with twice the memory took 10.9 ms there, 64 with half
+// 10.1; four n2 10.2, one 10.4; two or eight loads 10.7 and 11.1; runs that are
+// no multiple of 128 bytes 15 to 18.
+constexpr int kFinN2 = 2;
+constexpr int kFinU = 4;
+constexpr int kFinNJ = 8;
+constexpr int kFinBytes = 18 * 1024;
+constexpr int kFinThreads = 128;
+constexpr long long kFinBlocks = 12288;
 
-// Fallback for shapes whose (k1, m) plane does not fit in shared memory: one
-// thread per output entry of the n2 range, gathering from the accumulator.
-template <bool PAIR>
-__global__ void k_finalize_gather(const double2* __restrict__ acc, double inv_s,
-                                  double2* __restrict__ out, G4Dims d, int n2_0, int n2_cnt,
-                                  long long out_plane) {
-    const long long cnt = (long long)d.Nwex * n2_cnt * d.Nw2 * d.Nkex * d.Nc * d.Nc;
-    for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < cnt;
-         o += (long long)gridDim.x * blockDim.x) {
-        long long t = o;
-        const int k1 = (int)(t % d.Nc); t /= d.Nc;
-        const int k2 = (int)(t % d.Nc); t /= d.Nc;
-        const int q = (int)(t % d.Nkex); t /= d.Nkex;
-        const int n1 = (int)(t % d.Nw2); t /= d.Nw2;
-        const int n2l = (int)(t % n2_cnt);
-        const int m = (int)(t / n2_cnt);
-        const int n2 = n2_0 + n2l;
-        const size_t K1 = (size_t)k1 * d.Nw2 + n1, K2 = (size_t)k2 * d.Nw2 + n2;
-        const double2 v = acc_value<PAIR>(acc, (K1 * d.N + K2) * d.NQ + (size_t)q * d.Nwex + m);
-        const size_t po = (((size_t)n2l * d.Nw2 + n1) * d.Nkex + q) * d.Nc * d.Nc + (size_t)k2 * d.Nc + k1;
-        out[(size_t)m * out_plane + po] = make_double2(v.x * inv_s, v.y * inv_s);
+template <bool PAIR, bool DIRECT>
+__global__ void __launch_bounds__(kFinThreads) k_finalize(
+    const double2* __restrict__ acc, const float2* __restrict__ scr,
+    const double2* __restrict__ scr0, double inv_s, double2* __restrict__ out, G4Dims d, int TQ,
+    int RC, int nsplit, int n2_0, int n2_cnt, int q0, int nq, long long out_plane) {
+    extern __shared__ double2 tileF[];  // [kFinN2][RC][ld]
+    const int Nc = d.Nc, Nw2 = d.Nw2, Nwex = d.Nwex, NR = Nc * Nc;
+    const int n1 = blockIdx.x, n2b = blockIdx.y * kFinN2;
+    const int zq = blockIdx.z / nsplit, split = blockIdx.z - zq * nsplit, qb = zq * TQ;
+    const int NJ = min(TQ, nq - qb) * Nwex;          // transfers (q, m), contiguous in acc
+    const int nn = min(kFinN2, n2_cnt - n2b);
+    const int ld = NJ | 1;                           // odd: the transposed reads are conflict-free
+    const int L = NJ * kFinN2, G = kFinThreads / L;  // threads per momentum pair; pairs at a time
+    const int g = threadIdx.x / L, jn = threadIdx.x - g * L;
+    const int n2l = jn / NJ, j = jn - n2l * NJ;
+    const int n2 = n2_0 + n2b + n2l;
+    const bool mine = g < G && n2l < nn;
+    const int m = d.m0 + j % Nwex;
+    const int Ql = qb * Nwex + j;                    // plane of the group's scratch
+    const bool on = DIRECT && n1 + m < Nw2 && n2 + m < Nw2;   // else structurally zero
+    const bool first = q0 == 0 && Ql == 0;           // Q = 0: FP64 scratch
+    const size_t a1 = (size_t)Nw2 * d.N * d.NQ, a2 = (size_t)Nw2 * d.NQ;
+    const double2* ap = acc + ((size_t)n1 * d.N + n2) * d.NQ + (size_t)(q0 + qb) * Nwex + j;
+    const size_t s1 = (size_t)Nw2 * d.N, sofs = (size_t)n1 * d.N + n2;
+    const float2* sp = DIRECT ? scr + (size_t)Ql * d.N * d.N + sofs : nullptr;
+    const int dk2 = G / Nc, dk1 = G - dk2 * Nc;      // r += G
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int r0 = split * RC; r0 < NR; r0 += nsplit * RC) {
+        const int rc = min(RC, NR - r0);
+        if (mine) {
+            int k2 = (r0 + g) / Nc, k1 = r0 + g - k2 * Nc;
+            for (int rb = g; rb < rc; rb += kFinU * G) {
+                double2 v[kFinU];
+                float2 f[kFinU];
+                size_t f0[kFinU];
+#pragma unroll
+                for (int u = 0; u < kFinU; ++u) {
+                    if (rb + u * G < rc) {
+                        v[u] = acc_value<PAIR>(ap, (size_t)k1 * a1 + (size_t)k2 * a2);
+                        if constexpr (DIRECT) {
+                            f0[u] = (size_t)k1 * s1 + (size_t)(k2 * Nw2);
+                            if (on && !first) f[u] = sp[f0[u]];
+                        }
+                    }
+                    k1 += dk1;
+                    k2 += dk2;
+                    if (k1 >= Nc) {
+                        k1 -= Nc;
+                        ++k2;
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < kFinU; ++u) {
+                    const int rr = rb + u * G;
+                    if (rr >= rc) break;
+                    if constexpr (DIRECT) {
+                        if (on) {
+                            const double2 t = first ? scr0[f0[u] + sofs]
+                                                    : make_double2(g4ptx::f32_to_f64(f[u].x), g4ptx::f32_to_f64(f[u].y));
+                            v[u].x += t.x;
+                            v[u].y += t.y;
+                        }
+                    }
+                    tileF[((size_t)n2l * RC + rr) * ld + j] = v[u];
+                }
+            }
+        }
+        __syncthreads();
+        // a warp writes one (n2, q, m) plane's run of rc entries at a time
+        for (int pl = warp; pl < nn * NJ; pl += kFinThreads / 32) {
+            const int nl = pl / NJ, jj = pl - nl * NJ, qi = jj / Nwex, ml = jj - qi * Nwex;
+            double2* o = out + (size_t)ml * out_plane +
+                         (((size_t)(n2b + nl) * Nw2 + n1) * d.Nkex + q0 + qb + qi) * NR + r0;
+            const double2* t = tileF + (size_t)nl * RC * ld + jj;
+            for (int rr = lane; rr < rc; rr += 32) {
+                const double2 v = t[(size_t)rr * ld];
+                o[rr] = make_double2(v.x * inv_s, v.y * inv_s);
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -510,26 +563,25 @@ cudaError_t launch_update_fp64(const double2* G, const G4Signs& signs, int stage
 }
 
 cudaError_t launch_finalize(const double2* acc, bool pair, double inv_s, double2* out,
-                            const G4Dims& d, int n2_0, int n2_cnt, long long out_plane,
-                            cudaStream_t s) {
-    int KC = (int)((24 * 1024) / ((size_t)d.Nc * (d.Nwex + 1) * sizeof(double2)));
-    KC = KC < 1 ? 1 : (KC > d.Nc ? d.Nc : KC);
-    const size_t smem = (size_t)KC * d.Nc * (d.Nwex + 1) * sizeof(double2);
-    cudaError_t e;
-    if (smem > 96 * 1024) {
-        const long long cnt = (long long)d.Nwex * n2_cnt * d.Nw2 * d.Nkex * d.Nc * d.Nc;
-        long long blocks = (cnt + 255) / 256;
-        if (blocks > 152 * 64) blocks = 152 * 64;
-        auto* k = pair ? k_finalize_gather<true> : k_finalize_gather<false>;
-        k<<<(int)blocks, 256, 0, s>>>(acc, inv_s, out, d, n2_0, n2_cnt, out_plane);
-    } else {
-        auto* k = pair ? k_finalize<true> : k_finalize<false>;
-        if (smem > 48 * 1024) {
-            e = raise_smem_limit(k);
-            if (e != cudaSuccess) return e;
-        }
-        k<<<dim3(d.Nw2, n2_cnt, d.Nkex), 256, smem, s>>>(acc, inv_s, out, d, KC, n2_0, out_plane);
-    }
+                            const G4Dims& d, int n2_0, int n2_cnt, long long out_plane, int q0,
+                            int nq, const float2* scr, const double2* scr0, cudaStream_t s) {
+    // transfers per block: a 128-byte run, or one momentum's (NJ * kFinN2 is at
+    // most kFinThreads: Nwex <= 64)
+    const int TQ = std::min(nq, std::max(1, kFinNJ / d.Nwex));
+    const int NJ = TQ * d.Nwex, ld = NJ | 1;
+    const size_t per = (size_t)kFinN2 * ld * sizeof(double2);
+    int RC = (int)std::min<size_t>((size_t)d.Nc * d.Nc, std::max<size_t>(1, kFinBytes / per));
+    if (RC >= 8) RC = RC / 8 * 8;
+    // the chunks are dealt to enough blocks to fill the GPU several times over
+    // (8x8 cluster, 32 frequencies: 15.0 ms with a group's blocks undivided, 11.0
+    // divided)
+    const long long blocks = (long long)d.Nw2 * ((n2_cnt + kFinN2 - 1) / kFinN2) * ((nq + TQ - 1) / TQ);
+    const long long chunks = ((long long)d.Nc * d.Nc + RC - 1) / RC;
+    const int nsplit = (int)std::min<long long>(std::min<long long>(chunks, 256), (kFinBlocks + blocks - 1) / blocks);
+    const dim3 grid(d.Nw2, (n2_cnt + kFinN2 - 1) / kFinN2, (nq + TQ - 1) / TQ * nsplit);
+    auto* k = pair ? k_finalize<true, false> : scr ? k_finalize<false, true> : k_finalize<false, false>;
+    k<<<grid, kFinThreads, RC * per, s>>>(acc, scr, scr0, inv_s, out, d, TQ, RC, nsplit, n2_0, n2_cnt, q0, nq,
+                                          out_plane);
     return cudaGetLastError();
 }
 

@@ -546,7 +546,7 @@ struct DirectPlan {
     int fill = 0;        // measurements in the window
     int batches = 0;     // full batches the window holds
     int Kst = 0;         // row stride of the split planes (2 * Bw elements)
-    int nQg = 0;         // transfers per group
+    int nQg = 0;         // transfers per group (whole momenta where Nwex allows it)
     bool f16 = true;     // FP16 (else TF32) hi/lo planes
     float2* araw = nullptr;   // [NQ][N][Bw]
     float2* braw = nullptr;
@@ -620,7 +620,7 @@ g4_status direct_prepare(g4_ctx* h) {
     X->f16 = h->opt.operands == G4_OPERANDS_FP16;
     X->Bw = (F * h->batch + 31) / 32 * 32;   // 2 Bw: a whole number of 64-element stages
     X->Kst = 2 * X->Bw;
-    X->nQg = std::min(kGroupQ, d.NQ);
+    X->nQg = std::min(d.Nwex <= kGroupQ ? kGroupQ / d.Nwex * d.Nwex : kGroupQ, d.NQ);
     g4_status st;
     const size_t raw = (size_t)d.NQ * d.N * X->Bw;
     if ((st = dalloc(h, &X->araw, raw)) != G4_OK) return st;
@@ -668,7 +668,7 @@ int direct_window(const g4_ctx* h) {
     return X ? X->Bw : 0;
 }
 
-g4_status direct_pack(g4_ctx* h, int staged, bool* flush_due) {
+g4_status direct_pack(g4_ctx* h, int staged) {
     DirectPlan* X = (DirectPlan*)h->dplan;
     const G4Dims& d = h->d;
     if (X->fill + staged > X->Bw) return g4_fail(h, G4_ERR_STATE, "direct-term window overflow");
@@ -683,13 +683,15 @@ g4_status direct_pack(g4_ctx* h, int staged, bool* flush_due) {
         if (e != cudaSuccess) return g4_cuda_fail(h, e, "direct pack launch");
     }
     X->fill += staged;
-    *flush_due = X->fill + h->batch > X->Bw;
     return G4_OK;
 }
 
-g4_status direct_flush(g4_ctx* h) {
+namespace {
+// The window's GEMM, group by group into the scratch, and use(Q0, nQ) after
+// each group's.
+template <typename F>
+g4_status direct_groups(g4_ctx* h, F&& use) {
     DirectPlan* X = (DirectPlan*)h->dplan;
-    if (!X || X->fill == 0) return G4_OK;
     const G4Dims& d = h->d;
     const int Bwp = (X->fill + 31) / 32 * 32;
     DParams P;
@@ -726,18 +728,50 @@ g4_status direct_flush(g4_ctx* h) {
         gemm<<<grid, kThreads, kSmemBytes, h->stream>>>(X->mAh, X->mAl, X->mBh, X->mBl, P);
         prof_end(h, G4_K_DIRECT);
         if ((e = cudaGetLastError()) != cudaSuccess) return g4_cuda_fail(h, e, "direct launch");
+        const g4_status st = use(Q0, nQ);
+        if (st != G4_OK) return st;
+    }
+    return G4_OK;
+}
+
+}  // namespace
+
+g4_status direct_flush(g4_ctx* h) {
+    DirectPlan* X = (DirectPlan*)h->dplan;
+    if (!X || X->fill == 0) return G4_OK;
+    const G4Dims& d = h->d;
+    const g4_status st = direct_groups(h, [&](int Q0, int nQ) {
         prof_begin(h, G4_K_DIRECT_MERGE);
         auto* merge = h->opt.accum == G4_ACCUM_F32PAIR ? k_merge_pair : k_merge;
         merge<<<dim3((d.N + kMergeK2 - 1) / kMergeK2, d.N), 256, 0, h->stream>>>(
             X->scr, X->scr0, h->acc, Q0, nQ, d);
         prof_end(h, G4_K_DIRECT_MERGE);
-        if ((e = cudaGetLastError()) != cudaSuccess) return g4_cuda_fail(h, e, "direct merge launch");
-    }
+        cudaError_t e = cudaGetLastError();
+        return e == cudaSuccess ? G4_OK : g4_cuda_fail(h, e, "direct merge launch");
+    });
+    if (st != G4_OK) return st;
     // the next window's maximum starts again
-    if ((e = cudaMemsetAsync(X->wmax, 0, sizeof(unsigned), h->stream)) != cudaSuccess)
-        return g4_cuda_fail(h, e, "direct window maximum clear");
+    cudaError_t e = cudaMemsetAsync(X->wmax, 0, sizeof(unsigned), h->stream);
+    if (e != cudaSuccess) return g4_cuda_fail(h, e, "direct window maximum clear");
     X->fill = 0;
     return G4_OK;
+}
+
+bool direct_finalize_ok(const g4_ctx* h) {
+    const DirectPlan* X = (const DirectPlan*)h->dplan;
+    return X && X->fill > 0 && X->nQg % h->d.Nwex == 0 && h->opt.accum != G4_ACCUM_F32PAIR;
+}
+
+g4_status direct_finalize(g4_ctx* h, double inv_s, double2* out) {
+    const DirectPlan* X = (const DirectPlan*)h->dplan;
+    const G4Dims& d = h->d;
+    return direct_groups(h, [&](int Q0, int nQ) {
+        prof_begin(h, G4_K_FINALIZE);
+        cudaError_t e = launch_finalize(h->acc, false, inv_s, out, d, 0, d.Nw2, d.E / d.Nwex,
+                                        Q0 / d.Nwex, nQ / d.Nwex, X->scr, X->scr0, h->stream);
+        prof_end(h, G4_K_FINALIZE);
+        return e == cudaSuccess ? G4_OK : g4_cuda_fail(h, e, "finalize launch");
+    });
 }
 
 void direct_reset(g4_ctx* h) {

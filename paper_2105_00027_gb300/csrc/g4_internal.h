@@ -180,12 +180,14 @@ void f64tc_prepare(g4_ctx* h);
 bool f64tc_wanted(const g4_ctx* h, int staged);
 g4_status f64tc_run(g4_ctx* h, int staged);
 void f64tc_release(g4_ctx* h);
-// out = acc / S in the exported layout, for the n2 planes [n2_0, n2_0 + n2_cnt):
-// plane m of the block is written at out + m * out_plane (E / Nwex for the
-// whole array with n2_0 = 0, n2_cnt = 2Nw)
+// out = acc / S in the exported layout, for the n2 planes [n2_0, n2_0 + n2_cnt)
+// and the transfer momenta [q0, q0 + nq): plane m of the block is written at
+// out + m * out_plane (E / Nwex for the whole array with n2_0 = 0, n2_cnt =
+// 2Nw).  With scr given, (acc + scr) / S: the direct term's scratch planes
+// [nq * Nwex][K1][K2] of these momenta, FP64 in scr0 for Q = 0 (not for pairs)
 cudaError_t launch_finalize(const double2* acc, bool pair, double inv_s, double2* out,
-                            const G4Dims& d, int n2_0, int n2_cnt, long long out_plane,
-                            cudaStream_t s);
+                            const G4Dims& d, int n2_0, int n2_cnt, long long out_plane, int q0,
+                            int nq, const float2* scr, const double2* scr0, cudaStream_t s);
 // one measurement's G~ into its batch slot of Gd, its largest component
 // joining *gmax
 cudaError_t launch_build_G_diag(const void* M, bool m64, const double2* G0, double sign,
@@ -205,11 +207,15 @@ g4_status xtc_run(g4_ctx* h, int staged);
 void xtc_release(g4_ctx* h);
 
 // mixed-path direct term on tensor cores (g4_direct_tc.cu): operands of the
-// staged batch into the window (flush_due: the next batch would not fit),
-// and the window's GEMM added to the accumulator
+// staged batch into the window, and the window's GEMM added to the accumulator
+// (direct_flush, which empties the window) or to the exported result (
+// direct_finalize, which leaves both as they are; direct_finalize_ok: the
+// handle's transfers and accumulator allow it)
 g4_status direct_prepare(g4_ctx* h);
-g4_status direct_pack(g4_ctx* h, int staged, bool* flush_due);
+g4_status direct_pack(g4_ctx* h, int staged);
 g4_status direct_flush(g4_ctx* h);
+bool direct_finalize_ok(const g4_ctx* h);
+g4_status direct_finalize(g4_ctx* h, double inv_s, double2* out);
 void direct_reset(g4_ctx* h);
 int direct_fill(const g4_ctx* h);
 int direct_window(const g4_ctx* h);
