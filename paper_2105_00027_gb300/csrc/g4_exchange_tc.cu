@@ -239,7 +239,9 @@ struct PackM {
     static constexpr int SL = F16 ? 32 : 16;          // slots per spin and tile
     static constexpr int EB = M64 ? 8 : 16;           // bytes of an entry of M
     static constexpr int ET = M64 ? 128 : 64;         // entries per tile
-    static constexpr int THREADS = 512;
+    static constexpr int THREADS = 512;               // consumers
+    static constexpr int PROD = 128;                  // producers
+    static constexpr int CH = ET * EB / 16;           // 16-byte pieces of one slot's entries: 64
     static constexpr int QS = F16 ? 8 : 4;            // slots of a quarter (one 16-byte vector)
     static constexpr int QPAD = 32;                   // shift of each quarter group (bank spread)
     static constexpr int MBYTES = 2 * SL * ET * EB + (2 * SL / QS) * QPAD;  // M pieces of one stage
@@ -253,16 +255,17 @@ struct PackM {
     static constexpr int STAGE = MBYTES + GBYTES;     // bytes of one stage
     static constexpr int NST = 3;                     // stages
     static constexpr int MAXNC = 256;
-    // stages, D = 0 positions, slot sign factors, full and empty mbarriers, flag
-    static constexpr int SMEM = NST * STAGE + MAXNC * 4 + kMaxBatch * 8 + 2 * NST * 8 + 16;
+    // stages, D = 0 positions, slot sign factors, M pointers, full and empty mbarriers, flag
+    static constexpr int SMEM = NST * STAGE + MAXNC * 4 + kMaxBatch * 16 + 2 * NST * 8 + 16;
 };
 
-__device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(sdst)),
-        "l"(gsrc), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
+__device__ __forceinline__ void cp_async16(void* sdst, const void* gsrc) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(sdst)), "l"(gsrc) : "memory");
+}
+// Arrive on the barrier (one of its expected arrivals) once every copy this
+// thread has issued has landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // Deferred staging: the exchange operand planes (and, for channels with a
@@ -272,11 +275,11 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
 // rows of 2Nw < ET columns, or ET columns of one row), and SL consecutive
 // slots of both spins (SL = 32 FP16 or 16 TF32 values: a 64-byte half line of
 // an X row per spin).  Persistent, one block per SM, each block a contiguous
-// range of tiles (column momentum fastest).  A producer warp brings each
+// range of tiles (column momentum fastest).  Four producer warps bring each
 // tile's rows of M (one row piece per slot and spin) and, when every
 // measurement shares one G0, the G0 of the tile's rows and columns into a ring
-// of NST shared-memory stages with bulk copies that complete on the stage's
-// full mbarrier, refilling a stage when its empty mbarrier says the 16
+// of NST shared-memory stages with 16-byte asynchronous copies that arrive on the
+// stage's full mbarrier, refilling a stage when its empty mbarrier says the 16
 // consumer warps are done with it.  Consumers: four lanes per (entry, spin),
 // each a quarter of the slots, form G~ from the staged M and write the half
 // line of each plane and component of the row X[a(dk, dn)][k][n = j][c]
@@ -292,11 +295,17 @@ __device__ __forceinline__ void bulk_load(void* sdst, const void* gsrc, uint32_t
 // component, FP32 bits); the largest component formed joins *gmax_out when it
 // is given.  With redo != nullptr the launch does nothing unless *redo is set.
 // Every mbarrier wait is bounded: on timeout the block records
-// G4_DEV_TIMEOUT, waits (bounded) for the copies it issued and returns.  M and
+// G4_DEV_TIMEOUT, waits for the copies it issued and returns.
+// Bound by how fast one SM takes copies of M: with a producer warp issuing bulk
+// copies, one per row piece (256 of 256 bytes a tile at 32 frequencies), the
+// copies' number set the pace -- 128-byte instead of 64-byte stores, a branch-
+// free slot loop and conflict-free direct-term reads each changed nothing.  16
+// bytes per lane from four warps: 8x8 cluster, 32 frequencies, 128 slots 8.4 ->
+// 3.9 ms a pass (18 GB moved; a run of two batches 52.6 -> 43.6).  M and
 // G0 must be 16-byte aligned (checked when a deferred handle stages a
 // measurement).
 template <bool F16, bool M64>
-__global__ void __launch_bounds__(544, 1) k_pack_xtc_M(const __grid_constant__ G4SlotTable T, int staged,
+__global__ void __launch_bounds__(640, 1) k_pack_xtc_M(const __grid_constant__ G4SlotTable T, int staged,
                                                        int Jh, const float2* __restrict__ g0f,
                                                        const int* __restrict__ pos0g, int a0, int na,
                                                        void* __restrict__ Xh, void* __restrict__ Xl,
@@ -313,7 +322,8 @@ __global__ void __launch_bounds__(544, 1) k_pack_xtc_M(const __grid_constant__ G
     int* pos0 = reinterpret_cast<int*>(smem + NST * C::STAGE);
     float* srs = reinterpret_cast<float*>(pos0 + C::MAXNC);    // slot sign factors: magnitude
     int* sneg = reinterpret_cast<int*>(srs + kMaxBatch);         // and whether i times it
-    uint64_t* bar = reinterpret_cast<uint64_t*>(sneg + kMaxBatch);  // full[NST], then empty[NST]
+    const unsigned char** mptr = reinterpret_cast<const unsigned char**>(sneg + kMaxBatch);
+    uint64_t* bar = reinterpret_cast<uint64_t*>(mptr + kMaxBatch);  // full[NST], then empty[NST]
     uint64_t* ebar = bar + NST;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(ebar + NST);
     const int Nc = d.Nc, Nw2 = d.Nw2, N = d.N, Lx = d.Lx, Ly = d.Ly;
@@ -346,10 +356,11 @@ __global__ void __launch_bounds__(544, 1) k_pack_xtc_M(const __grid_constant__ G
     for (int t = tid; t < staged; t += blockDim.x) {
         srs[t] = T.s[t].rs;
         sneg[t] = T.s[t].neg;
+        mptr[t] = reinterpret_cast<const unsigned char*>(T.s[t].M);
     }
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
-            mbar_init(&bar[s], 1);
+            mbar_init(&bar[s], C::PROD);
             mbar_init(&ebar[s], C::THREADS / 32);
         }
         *abort_flag = 0;
@@ -423,40 +434,38 @@ __global__ void __launch_bounds__(544, 1) k_pack_xtc_M(const __grid_constant__ G
     };
     const long long t_begin = (long long)blockIdx.x * ntiles / gridDim.x;
     const long long t_end = (long long)(blockIdx.x + 1) * ntiles / gridDim.x;
-    // producer warp: the copies of tile c into stage s -- one row piece of M
-    // per live slot, spin and row, and (shared G0) the complex64 G0 rows of the
-    // tile's two momenta for both spins
+    // producers: the copies of tile c into stage s -- the live slots' entries of M
+    // and (shared G0) the complex64 G0 rows of the tile's two momenta for both
+    // spins.  A producer keeps its 16-byte piece w of a slot's ET entries (rows
+    // of CJ) and takes every PROD / CH-th slot.
+    const int pt = tid - C::THREADS;
+    const int w = pt & (C::CH - 1), cpr = CJ * EB / 16;
+    const int wrow = w / cpr, wcol = w - wrow * cpr;
     auto issue = [&](const Tile& c, int s) {
         const Geo g = geo(c);
         const int nlive = max(0, min(SL, staged - g.r0));
-        const int ncopy = 2 * nlive * g.ri;
-        const uint32_t piece = (uint32_t)g.cj * EB;
         unsigned char* st = smem + (size_t)s * C::STAGE;
-        const uint32_t gbytes = g0f ? 4u * (uint32_t)Nw2 * 8u : 0u;
-        if ((tid & 31) == 0) {
-            const uint32_t bytes = (uint32_t)ncopy * piece + gbytes;
-            if (bytes > 0) mbar_expect_tx(&bar[s], bytes);
-            else mbar_arrive(&bar[s]);
+        if (wrow < g.ri && wcol * 16 < g.cj * EB) {
+            const size_t off = ((size_t)(g.kr * Nw2 + g.i0 + wrow) * N + g.k * Nw2 + g.j0) * EB + 16 * wcol;
+#pragma unroll
+            for (int ss = 0; ss < 2; ++ss)
+#pragma unroll 8
+                for (int us = pt / C::CH; us < nlive; us += C::PROD / C::CH)
+                    cp_async16(st + C::moff(ss, us, 0) + 16 * w, mptr[g.r0 + us] + ss * NN * EB + off);
         }
-        __syncwarp();
-        for (int c = tid & 31; c < ncopy; c += 32) {
-            const int row = c % g.ri, rest = c / g.ri;
-            const int us = rest % nlive, ss = rest / nlive;
-            const unsigned char* src = reinterpret_cast<const unsigned char*>(T.s[g.r0 + us].M) +
-                                       ((size_t)ss * NN + (size_t)(g.kr * Nw2 + g.i0 + row) * N +
-                                        g.k * Nw2 + g.j0) * EB;
-            bulk_load(st + C::moff(ss, us, row * CJ), src, piece, &bar[s]);
-        }
-        if (g0f && (tid & 31) < 4) {
+        if (g0f) {
             // [spin][0: row momentum kr | 1: column momentum k][2Nw] complex64
-            const int z = (tid & 31) >> 1, col = (tid & 31) & 1;
-            const float2* src = g0f + (size_t)z * N + (size_t)(col ? g.k : g.kr) * Nw2;
-            bulk_load(st + C::MBYTES + (size_t)(z * 2 + col) * Nw2 * 8, src, (uint32_t)Nw2 * 8u, &bar[s]);
+            for (int q = pt; q < 2 * Nw2; q += C::PROD) {
+                const int z = q / (Nw2 / 2), col = q - z * (Nw2 / 2);
+                const float2* src = g0f + (size_t)(z >> 1) * N + (size_t)(z & 1 ? g.k : g.kr) * Nw2 + 2 * col;
+                cp_async16(st + C::MBYTES + (size_t)z * Nw2 * 8 + 16 * col, src);
+            }
         }
+        cp_async_arrive(&bar[s]);
     };
     float vmax = 0.f, dmax = 0.f;
     if (tid >= C::THREADS) {
-        // producer warp: refill each stage once its consumer warps have released it
+        // producers: refill each stage once its consumer warps have released it
         int it = 0;
         Tile c = tile_at(t_begin);
         for (long long tt = t_begin; tt < t_end; ++tt, ++it, tile_next(c)) {
@@ -464,13 +473,9 @@ __global__ void __launch_bounds__(544, 1) k_pack_xtc_M(const __grid_constant__ G
             if (it >= NST && !mbar_wait(&ebar[s], (uint32_t)(it / NST - 1) & 1u, budget, abort_flag)) break;
             issue(c, s);
         }
-        // no copy may be in flight when the block exits: wait (bounded) for
-        // the last tiles issued (their copies have normally landed already)
-        if ((tid & 31) == 0) {
-            for (int k2 = 1; k2 <= NST && it - k2 >= 0; ++k2)
-                mbar_drain(&bar[(it - k2) % NST], (uint32_t)((it - k2) / NST) & 1u, kDrainBudget);
-            if (*abort_flag) atomicOr(status, (unsigned)G4_DEV_TIMEOUT);
-        }
+        // no copy may be in flight when the block exits
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if ((tid & 31) == 0 && *abort_flag) atomicOr(status, (unsigned)G4_DEV_TIMEOUT);
         return;
     }
     int it = 0;
@@ -602,7 +607,7 @@ __global__ void __launch_bounds__(544, 1) k_pack_xtc_M(const __grid_constant__ G
         __syncwarp();
         if ((tid & 31) == 0) mbar_arrive(&ebar[s]);
     }
-    if (*abort_flag) return;  // the producer waits for its copies
+    if (*abort_flag) return;  // the producers wait for their copies
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
@@ -1672,7 +1677,7 @@ g4_status xtc_run(g4_ctx* h, int staged) {
             }
             const int passes = X->f16 && !first ? 2 : 1;
             for (int pass = 0; pass < passes && e == cudaSuccess; ++pass) {
-                pack<<<X->packm_grid, 544, smem, h->stream>>>(
+                pack<<<X->packm_grid, 640, smem, h->stream>>>(
                     *h->slots, staged, X->Jh, g0s ? X->g0f : nullptr, X->pos0, X->gd0[g], X->gdn[g], X->Xh, X->Xl,
                     h->gscale, pass == 0 && passes == 2 ? h->gmax : nullptr, pass ? h->gredo : nullptr, D, d,
                     P.budget, h->dstatus);
