@@ -449,8 +449,7 @@ __global__ void __launch_bounds__(256) k_build_G_diag(const void* __restrict__ M
     const int c = blockIdx.x * kDiagCols + lane, kr = blockIdx.y, sp = blockIdx.z;
     const bool ok = c < N;
     // M and G0 may come from the kernel before: nothing is read until it is done
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    g4ptx::pdl_wait();
     const MV* src = reinterpret_cast<const MV*>(M) + ((size_t)sp * N + (size_t)kr * Nw2) * N + c;
     if (ok)
         for (int i = warp; i < Nw2; i += nwarp)
@@ -598,15 +597,5 @@ cudaError_t launch_build_G_diag(const void* M, bool m64, const double2* G0, doub
     }
     // a run is a chain of these launches: the next one's blocks are set up while
     // this one finishes, and wait for it (on the device) before their first read
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, M, G0, g4gt::sign_factor(sign), Gd_slot, ksub, d, gmax);
+    return launch_pdl(k, grid, dim3(256), smem, s, M, G0, g4gt::sign_factor(sign), Gd_slot, ksub, d, gmax);
 }

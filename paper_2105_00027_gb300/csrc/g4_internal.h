@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "g4.h"
@@ -72,6 +73,25 @@ inline cudaError_t raise_smem_limit(F* fn) {
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 optin - (int)fa.sharedSizeBytes);
+}
+
+// Launch with programmatic stream serialisation: the grid's blocks are set up
+// while the kernel before it finishes.  The kernel calls pdl_wait before its
+// first access to global memory, so the order of a plain launch is kept; a
+// chain of small kernels saves about 2 us per launch.
+template <typename... K, typename... A>
+inline cudaError_t launch_pdl(void (*k)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... a) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, std::forward<A>(a)...);
 }
 
 struct g4_ctx {

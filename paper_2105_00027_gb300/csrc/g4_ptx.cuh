@@ -212,6 +212,13 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
+// Start of a kernel launched by launch_pdl: let the next kernel's blocks be set
+// up, and wait until the kernel before has completed and its writes are seen.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // FP32 -> FP64 widening on the integer pipes.  GB300's FP64 pipe is narrow:
 // an epilogue that widens every accumulator value with cvt.f64.f32 is bound by
 // it, so the epilogues widen half of their values here and half in hardware.
