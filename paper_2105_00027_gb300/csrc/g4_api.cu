@@ -21,7 +21,7 @@ std::atomic<unsigned long long> g_next_uid{1};
 
 // Executable graphs of g4_accumulate_group, one per group signature: the
 // handles (by identifier) in launch order, the number of measurements each had
-// staged and how full its direct-term window was (which decides where the
+// staged, whether its accumulator was still to be written and how full its direct-term window was (which decides where the
 // batch's operands go and whether the window is added).  While a group's
 // batches keep that shape the graph is relaunched as it is, and each handle's
 // window then advances as it did when the graph was captured; a destroyed
@@ -29,8 +29,9 @@ std::atomic<unsigned long long> g_next_uid{1};
 struct GroupKey {
     unsigned long long uid;
     int staged, fill;
+    bool fresh;   // the batch writes the accumulator instead of adding to it
     bool operator==(const GroupKey& o) const {
-        return uid == o.uid && staged == o.staged && fill == o.fill;
+        return uid == o.uid && staged == o.staged && fill == o.fill && fresh == o.fresh;
     }
 };
 struct GroupGraph {
@@ -159,6 +160,14 @@ g4_status accumulate_mixed(g4_ctx* h) {
     if (st == G4_OK) st = direct_pack(h, h->staged);
     if (st == G4_OK && !h->deferred) st = exchange_term(h);
     return st;
+}
+
+// Clear an accumulator that no batch has written.
+g4_status clear_fresh(g4_ctx* h) {
+    if (!h->fresh) return G4_OK;
+    G4_CUDA(h, cudaMemsetAsync(h->acc, 0, (size_t)h->d.E * sizeof(double2), h->stream));
+    h->fresh = false;
+    return G4_OK;
 }
 
 g4_status do_accumulate(g4_ctx* h) {
@@ -412,7 +421,11 @@ g4_status g4_create(int Nc, int Nw, int Nwex, int Nkex, g4_channel ch, const g4_
 
 g4_status g4_reset(g4_handle h) {
     if (!h) return G4_ERR_INVALID;
-    G4_CUDA(h, cudaMemsetAsync(h->acc, 0, (size_t)h->d.E * sizeof(double2), h->stream));
+    h->fresh = true;
+    if (!h->xtc || h->opt.accum == G4_ACCUM_F32PAIR) {
+        g4_status st = clear_fresh(h);
+        if (st != G4_OK) return st;
+    }
     G4_CUDA(h, cudaMemsetAsync(h->dstatus, 0, kStatusWords * sizeof(unsigned), h->stream));
     direct_reset(h);
     h->scaled = false;
@@ -494,7 +507,7 @@ g4_status g4_accumulate_group(g4_handle* hs, int n) {
     const cudaStream_t main = h0->stream;  // may be the legacy stream, which cannot capture
     const int nb = (int)work.size();
     std::vector<GroupKey> key;
-    for (g4_ctx* h : work) key.push_back(GroupKey{h->uid, h->staged, direct_fill(h)});
+    for (g4_ctx* h : work) key.push_back(GroupKey{h->uid, h->staged, direct_fill(h), h->fresh});
     {
         // a group shape seen before: relaunch its graph
         std::lock_guard<std::mutex> lock(g_graph_mu);
@@ -504,6 +517,7 @@ g4_status g4_accumulate_group(g4_handle* hs, int n) {
                 if (e != cudaSuccess) return g4_cuda_fail(h0, e, "grouped accumulate graph launch");
                 for (size_t i = 0; i < work.size(); ++i) {
                     work[i]->staged = 0;
+                    work[i]->fresh = false;
                     direct_set_fill(work[i], gg.fill_after[i]);
                 }
                 return G4_OK;
@@ -578,6 +592,7 @@ g4_status g4_finalize(g4_handle h, void* out, double* sign_sum) {
     if (!out) return g4_fail(h, G4_ERR_INVALID, "out is NULL");
     if (h->finalized) return g4_fail(h, G4_ERR_STATE, "g4_finalize called twice");
     g4_status st = do_accumulate(h);
+    if (st == G4_OK) st = clear_fresh(h);
     if (st != G4_OK) return st;
     cudaPointerAttributes attr;
     cudaError_t e = cudaPointerGetAttributes(&attr, out);
@@ -663,6 +678,7 @@ constexpr size_t kIoChunk = (size_t)256 << 20;
 g4_status g4_checkpoint(g4_handle h, const char* path) {
     if (!h || !path) return G4_ERR_INVALID;
     g4_status st = do_accumulate(h);
+    if (st == G4_OK) st = clear_fresh(h);
     if (st != G4_OK) return st;
     if (h->finalized && (st = direct_flush(h)) != G4_OK) return st;
     if ((st = sync_and_check(h)) != G4_OK) return st;
@@ -743,6 +759,10 @@ g4_status g4_restore(g4_handle h, const char* path) {
     } catch (...) {
         std::fclose(f);
         return g4_fail(h, G4_ERR_OOM, "host buffer for restore");
+    }
+    if (clear_fresh(h) != G4_OK) {
+        std::fclose(f);
+        return G4_ERR_CUDA;
     }
     cudaError_t e = cudaStreamSynchronize(h->stream);
     bool ok = e == cudaSuccess;

@@ -116,6 +116,8 @@ struct g4_ctx {
     // measurement (the mixed path adds the direct term once per window of
     // batches, see g4_direct_tc.cu); the exported result is acc / sum_r s_r
     double2* acc = nullptr;
+    bool fresh = false;              // acc is not cleared yet: the next batch of the tensor-core
+                                     // exchange writes it (any other use clears it first)
     unsigned* dstatus = nullptr;     // device status word
     unsigned* gmax = nullptr;        // largest |G~| component of the staged batch (FP32 bits),
                                      // for the FP16 operand scale; right after dstatus
