@@ -81,10 +81,14 @@ typedef enum {
     G4_PREC_FP64 = 0,      /* FP64 G and an update of FP64 accuracy, added to the
                               accumulator once per batch: plain FP64 kernels, or for
                               large batches (Nwex <= 16) on tensor cores, exact products
-                              of operands split into 54-bit integers' digits.  The
-                              latter keeps up to an eighth of the device memory free at
-                              g4_create, at most 8 GB, for its operands and is not used
-                              with mem_limit or timeout_cycles */
+                              of operands split into 62-bit integers' digits.  A batch
+                              with a G entry of which more than a quarter of the values
+                              of one spin lie more than 2^7 below the entry's largest
+                              value, or are outside 2^+-380, takes the plain kernels
+                              (the digits' error is relative to the largest value).  The
+                              tensor-core form keeps up to an eighth of the device memory
+                              free at g4_create, at most 8 GB, for its operands and is
+                              not used with mem_limit or timeout_cycles */
     G4_PREC_MIXED = 1      /* batched path: complex64 G, exchange-type term on tensor
                               cores (3-term FP16 or TF32 split, FP32 accumulate) or FP32
                               CUDA cores, added to the FP64 accumulator once per batch;

@@ -1,32 +1,44 @@
-// The FP64 path's update of a whole batch on the tcgen05 tensor cores, exact
-// to below FP64 rounding.
+// The FP64 path's update of a whole batch on the tcgen05 tensor cores, to FP64
+// accuracy.
 //
 // GB300's FP64 pipe issues two lanes per clock and SM: the twelve fused
 // multiply-adds of an element-update bound a plain FP64 kernel at 5e10
 // updates/s, whatever the memory system does.  The tensor cores reach FP64
-// precision through integer arithmetic instead: every operand becomes seven
-// signed base-256 digits of a 54-bit integer scaled by one power of two per
+// precision through integer arithmetic instead: every operand becomes eight
+// signed base-256 digits of a 62-bit integer scaled by one power of two per
 // operand row, each digit an FP16 value in [-128, 127] (exact), and the digit
 // products are summed in FP32 accumulators that never leave the integers below
 // 2^24 -- so every sum is exact.  (The error-free splitting of a matrix product
 // into slices with exact partial products is the method of Ozaki, Ogita, Oishi
 // and Rump, Numerical Algorithms 59, 2012.)
 //
-//   x = 2^(e-54) v,  |v| < 2^54,  v = sum_t d_t 256^(6-t),  t = 0..6
-//   u w = 2^(eu+ew-108) sum_p 256^(12-p) sum_{s+t=p} d_s(u) d_t(w)
+//   x = 2^(e-62) v,  |v| < 2^62,  v = sum_t d_t 256^(7-t),  t = 0..7
+//   u w = 2^(eu+ew-124) sum_p 256^(14-p) sum_{s+t=p} d_s(u) d_t(w)
 //
-// Levels p = 0..6 (28 digit products) are kept, each in its own accumulator;
-// the dropped ones are below 2^-55 of the product of the two rows' largest
-// values.  With at most 256 terms of K (64 measurements x 2 spins x 2
-// components) levels 0..4 stay below 2^24 whatever the digits are (the leading
-// digit is at most 64); levels 5 and 6, whose unit is 2^-52 and 2^-60 of that
-// product, could pass 2^24 only if nearly all of 1500 digit products were
-// largest and of one sign, and would then round to even integers.  The epilogue
-// puts the seven integers together in 64-bit integer arithmetic and rounds once
-// to FP64, off the FP64 pipe.  e is chosen per operand row (one G entry over the batch's
-// measurements and spins), so the range of G over momenta and frequencies
-// costs no digits.  A batch with a non-finite G entry, or a component outside
-// 2^+-380, is left to the plain kernels (a device flag set by the G build).
+// Levels p = 0..7 (36 digit products) are kept, each in its own accumulator.
+// With at most 256 terms of K (64 measurements x 2 spins x 2 components) levels
+// 0..4 stay below 2^24 whatever the digits are (the leading digit is at most
+// 64); levels 5 to 7, whose unit is 2^-52 of the largest product and less,
+// could pass 2^24 only if nearly all of 1500 digit products were largest and of
+// one sign, and would then round to even integers.  The epilogue puts the eight
+// integers together in 96-bit integer arithmetic and rounds once to FP64.
+//
+// Accuracy.  An operand is exact down to 2^-62 of its row's unit 2^e (the row:
+// one G entry over the batch's measurements and spins, real and imaginary part;
+// |x| < 2^e), and the dropped levels are below 2^-59 of 2^(eu+ew), 2^-62 in the
+// mean: an entry's error is relative to the rows' largest values, where FP64's
+// is relative to the products that are summed.  A pass over the staged G before
+// the first operand is formed (k_spread) keeps the two together: a batch with a
+// row of which more than a quarter of one spin's values lie more than 2^7 below
+// the row's largest is left to the plain kernels, as is one with a non-finite G
+// entry or a component outside 2^+-380 (one device flag for all of them).  What
+// remains has, for half of an entry's products or more, both factors above 2^-8
+// of their rows' units, which bounds the error by 2^-40 of the sum of the
+// products' moduli, all errors of one sign and all products as small as the
+// rule allows.  In the mean, of 128 products, relative to that sum: 4e-19 for
+// values of like size (a plain FP64 sum: 4e-17), 1e-16 for one value in each
+// row 2^6 above the others, in different measurements (plain: 2e-16).  Seven
+// digits and levels without such a check had 1e-16 and 4e-14, and no bound.
 //
 // The GEMMs are those of the mixed path (g4_exchange_tc.cu, g4_direct_tc.cu):
 //   exchange  rows K1 of diagonal D x columns P of diagonal -D, K = (r, spin)
@@ -40,19 +52,20 @@
 // 10.6 ms a batch on the 4x4 cluster with 64 frequencies and 8 transfers).
 //
 // k_gemm_digits, one CTA per SM, warp roles:
-//   warp 0      TMA producer: per 32 values of K one stage of 7 + 7 boxes
-//   warp 1      MMA issuer: per stage 28 products x 2 steps of 16 values of K,
-//               level by level; seven accumulators of up to 64 columns
+//   warp 0      TMA producer: per 32 values of K one stage of 8 + 8 boxes
+//   warp 1      MMA issuer: per stage 36 products x 2 steps of 16 values of K,
+//               level by level; eight accumulators of up to 64 columns
 //   warps 2..17 epilogue: four per tensor-memory lane quarter, each a quarter
 //               of the columns.  A level is drained into integer registers as
 //               soon as it is complete and handed back, while the next levels
 //               are still being multiplied.
 // What bounds it: the MMAs, whose 128-row A operand is read from shared memory
 // every time (128 x 64 x 16 per MMA: about 48 clocks of shared-memory reads for
-// 32 of arithmetic); seven accumulators of 64 columns fill tensor memory, so N
+// 32 of arithmetic); eight accumulators of 64 columns fill tensor memory, so N
 // cannot be larger; with few values of K the epilogue.  Measured, one batch of
 // 64 on the 4x4 cluster with 64 frequencies, 8 x 16 transfers: the plain tiled
-// kernel 279 ms; here 13 ms (exchange 6.8, direct 2.0, packs 2.5, merge 1.4).
+// kernel 279 ms; here 16 ms (exchange 8.5, direct 2.8, packs and spread 3.0,
+// merge 1.7).
 // Every wait is bounded as in the mixed path's kernels.
 #include <cudaTypedefs.h>
 #include <cuda_fp16.h>
@@ -71,7 +84,7 @@ namespace {
 
 using namespace g4ptx;
 
-constexpr int kDig = 7;                        // base-256 digits of an operand
+constexpr int kDig = 8;                        // base-256 digits of an operand
 constexpr int kChunk = 32;                     // K values per stage (64-byte rows)
 constexpr int kStages = 2;
 constexpr int kARows = 128;
@@ -81,9 +94,10 @@ constexpr int kEpiWarps = 16;
 constexpr int kThreads = 32 * (2 + kEpiWarps);
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMaxChunks = 8;
-constexpr int kRowEnt = 48;                    // most entries (pb Nwex) of a row's run buffer
 constexpr int kMaxWex = 16;                    // largest Nwex of this path
 constexpr int kMinSmem = 116 * 1024;           // two blocks never share an SM (tensor memory)
+constexpr int kMaxSmem = 227 * 1024;
+constexpr int kSpread = 7;                     // bits of spread within a row, see k_spread
 
 struct FSigns {
     double rs[64];          // sqrt(|s|)
@@ -91,16 +105,15 @@ struct FSigns {
 };
 
 // ------------------------------------------------------------------ digits
-// |x| < 2^e as v = round(x 2^(54-e)) on the integer pipes.
+// |x| < 2^e as v = round(x 2^(62-e)) on the integer pipes.
 __device__ __forceinline__ long long to_fixed(double x, int e) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int eb = (int)((b >> 52) & 0x7FFu);
     if (eb == 0) return 0;
     const unsigned long long mant = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const int sh = eb - 1021 - e;   // v = mant 2^sh, sh <= 1
+    const int sh = eb - 1013 - e;   // v = mant 2^sh, sh <= 9
     unsigned long long v;
-    if (sh > 0) v = mant << 1;
-    else if (sh == 0) v = mant;
+    if (sh >= 0) v = mant << sh;
     else if (sh <= -55) v = 0;
     else v = (mant + (1ull << (-sh - 1))) >> -sh;
     return (long long)b < 0 ? -(long long)v : (long long)v;
@@ -133,14 +146,14 @@ __device__ __forceinline__ void write_digits(const double* xs, int ld, int J, in
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const unsigned long long w =
-                (unsigned long long)(to_fixed(x[u], e) + 0x0080808080808080ll);
+                (unsigned long long)to_fixed(x[u], e) + 0x8080808080808080ull;
             lo[u] = (uint32_t)w;
             hi[u] = (uint32_t)(w >> 32);
         }
         __half* o = out + (size_t)(1 + c) * J + 4 * j;
 #pragma unroll
         for (int t = 0; t < kDig; ++t) {
-            // byte 6-t of two values into the low bytes of two halves: 1024 + b
+            // byte 7-t of two values into the low bytes of two halves: 1024 + b
             const int by = kDig - 1 - t, n = by & 3;
             const uint32_t sel = (uint32_t)(n | (n << 4) | ((4 + n) << 8) | ((4 + n) << 12));
             const uint32_t p01 = (__byte_perm(by < 4 ? lo[0] : hi[0], by < 4 ? lo[1] : hi[1], sel) & 0x00FF00FFu) | 0x64006400u;
@@ -157,15 +170,67 @@ __device__ __forceinline__ void write_digits(const double* xs, int ld, int J, in
     }
 }
 
+// Sets *flag when the digits would lose more than FP64 does (see the top of the
+// file): a G entry (i, j) -- a row of the exchange operands, and where it is
+// one of the direct operands (|n_i - n_j| a transfer of the handle) the spins'
+// combination -- of which more than a quarter of the values of one spin lie
+// more than 2^kSpread below the row's largest.  Zeros count as small, a row of
+// zeros alone does not.  One thread per entry; the exponents of its values are
+// kept in shared memory between the search for the largest and the count.
+// Bound by HBM (the staged G read once).
+struct SpreadArgs {
+    signed char se[64];   // exponent of a measurement's sign factor; -128: weight zero
+};
+
+__global__ void __launch_bounds__(256) k_spread(const double2* __restrict__ G, int staged,
+                                                const __grid_constant__ SpreadArgs A, bool direct, G4Dims d,
+                                                unsigned* __restrict__ flag) {
+    if (*flag) return;
+    extern __shared__ unsigned short exps[];   // [3 staged][256]: spin up, spin down, combination
+    const size_t NN = (size_t)d.N * d.N;
+    const double ws = d.ch == G4_PH_DENSITY ? 1.0 : -1.0;
+    unsigned short* ex = exps + threadIdx.x;
+    bool bad = false;
+    for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < NN; e += (size_t)gridDim.x * 256) {
+        const int i = (int)(e / d.N), j = (int)(e - (size_t)i * d.N);
+        const int dn = abs(i % d.Nw2 - j % d.Nw2);
+        const bool both = direct && dn >= d.m0 && dn < d.m0 + d.Nwex;
+        int top = 0, topd = 0;
+        auto put = [&](int row, double2 v, int se) {
+            const unsigned h = max((unsigned)__double2hiint(v.x) & 0x7FFFFFFFu,
+                                   (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu) >> 20;
+            const int x = h && se > -128 ? max((int)h + se, 1) : 0;
+            ex[row * 256] = (unsigned short)x;
+            return x;
+        };
+#pragma unroll 4
+        for (int r = 0; r < staged; ++r) {
+            const double2 a = G[(size_t)(2 * r) * NN + e], b = G[(size_t)(2 * r + 1) * NN + e];
+            const int se = A.se[r];
+            top = max(top, max(put(2 * r, a, se), put(2 * r + 1, b, se)));
+            if (both) topd = max(topd, put(2 * staged + r, make_double2(a.x + ws * b.x, a.y + ws * b.y), se));
+        }
+        int c0 = 0, c1 = 0, cd = 0;
+        for (int r = 0; r < staged; ++r) {
+            c0 += (int)ex[2 * r * 256] < top - kSpread;
+            c1 += (int)ex[(2 * r + 1) * 256] < top - kSpread;
+            if (both) cd += (int)ex[(2 * staged + r) * 256] < topd - kSpread;
+        }
+        if (top > 0 && max(c0, c1) > staged / 4) bad = true;
+        if (topd > 0 && cd > staged / 4) bad = true;
+    }
+    if (bad) *flag = 1u;
+}
+
 // Exchange operands of one group of diagonals [a0, a0 + na): every G entry
 // (i, j) as a row of J = 2 Jh values jj = spin * Jh + r per component, digit
-// planes X[(a * 7 + t)][k][n][c][jj], c = (-Im, Re, Im) (a: the group's position of the diagonal
+// planes X[(a * 8 + t)][k][n][c][jj], c = (-Im, Re, Im) (a: the group's position of the diagonal
 // (kr (-) k, ni - n) for i = (kr, ni), j = (k, n)) and exponents ex[a][k][n].
 // A block takes one row i and eight consecutive columns j of one momentum: it
 // reads one 128-byte line of every slot and spin, and writes whole rows of X
 // (2 J bytes per digit and component).  Values r >= staged are zero, written
 // up to the next multiple of 32 (the GEMM's chunks of K).  HBM-bound: 16 B
-// read and 42 B written per entry, slot and spin.
+// read and 48 B written per entry, slot and spin.
 constexpr int kPackJ = 8;
 
 __global__ void __launch_bounds__(256) k_pack_digits(const double2* __restrict__ G, int staged, int Jh,
@@ -222,7 +287,7 @@ __global__ void __launch_bounds__(256) k_pack_digits(const double2* __restrict__
 }
 
 // Direct operands of the transfers Q0 .. Q0 + gridDim.y: a_r(K) (side 0) and
-// b_r(K) (side 1) as digit planes P[side][(Ql * 7 + t)][K][c][r], r < Bp, c as above, and
+// b_r(K) (side 1) as digit planes P[side][(Ql * 8 + t)][K][c][r], r < Bp, c as above, and
 // exponents ex[side][Ql][K].  One block per eight frequencies of one momentum.
 __global__ void __launch_bounds__(256) k_pack_digits_ab(const double2* __restrict__ G, int staged, int Bp,
                                                         int live, FSigns sg, int Q0, int nQg,
@@ -287,18 +352,14 @@ struct FParams {
     long long budget;
 };
 
-// 16 consecutive 32-bit columns of this thread's lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
-        "%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-          "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-          "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
+// 8 consecutive 32-bit columns of this thread's lane.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
 #pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
 // Shared-memory matrix descriptor: K-major, 64-byte swizzle, 8-row atoms of
@@ -337,14 +398,33 @@ __device__ __forceinline__ bool quarter_any(int quad, bool p) {
     return r != 0;
 }
 
-// v 2^sc, rounded to nearest even (|sc| small enough for a normal result),
-// negated when neg is set.  One conversion on the FP64 pipe; scale and sign on
-// the integer pipes (the conversion there as well, about 45 instructions, made
-// the epilogue the limit of small batches).
-__device__ __forceinline__ double fixed_to_f64(long long v, int sc, bool neg) {
+// (hi, mid, lo) += w 2^(56-8p), level p's part of a 96-bit integer.  Shifts and
+// carries: 64-bit multiply-adds took the direct GEMM of one batch on the 4x4
+// cluster with 64 frequencies from 2.8 to 3.3 ms.
+template <int P>
+__device__ __forceinline__ void add_level(uint32_t& lo, uint32_t& mid, uint32_t& hi, int w) {
+    constexpr int S = 24 - 8 * (P & 3);
+    const uint32_t a = (uint32_t)w << S, b = (uint32_t)(w >> (S ? 32 - S : 31));
+    if constexpr (P < 4)
+        asm("add.cc.u32 %0, %0, %2;\n addc.u32 %1, %1, %3;" : "+r"(mid), "+r"(hi) : "r"(a), "r"(b));
+    else
+        asm("add.cc.u32 %0, %0, %3;\n addc.cc.u32 %1, %1, %4;\n addc.u32 %2, %2, %5;"
+            : "+r"(lo), "+r"(mid), "+r"(hi)
+            : "r"(a), "r"(b), "r"((uint32_t)(w >> 31)));
+}
+
+// (hi, mid, lo) 2^sc in FP64, rounded to nearest (|sc| small enough for a
+// normal result), negated when neg is set: the 64 leading bits (|t| < 2^78) go
+// through one conversion on the FP64 pipe; what is cut off is below 2^-61 of
+// the value.  Scale and sign on the integer pipes (the conversion there as
+// well, about 45 instructions, made the epilogue the limit of small batches).
+__device__ __forceinline__ double fixed_to_f64(uint32_t lo, uint32_t mid, uint32_t hi, int sc, bool neg) {
+    const long long h = (long long)(((unsigned long long)hi << 32) | mid);
+    const int s = min(32, __clzll(h ^ (h >> 63)) - 1);   // 17 .. 32
+    const long long v = (long long)(((unsigned long long)h << s) | (lo >> (32 - s)));
     const double x = __ll2double_rn(v);
-    const int hi = (__double2hiint(x) + sc * (1 << 20)) ^ (neg ? (int)0x80000000u : 0);
-    return v == 0 ? 0.0 : __hiloint2double(hi, __double2loint(x));
+    const int xh = (__double2hiint(x) + (sc + 32 - s) * (1 << 20)) ^ (neg ? (int)0x80000000u : 0);
+    return v == 0 ? 0.0 : __hiloint2double(xh, __double2loint(x));
 }
 
 struct FTile {
@@ -397,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t* tmem_slot = (uint32_t*)(mdone + 1);
     volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
     int* ebs = (int*)(smem + kStages * stage_bytes + 256);          // [4][kMaxN] column exponents
-    double* bufs = (double*)(ebs + 4 * kMaxN);                       // [4][16][kRowEnt + 1] complex
+    double* bufs = (double*)(ebs + 4 * kMaxN);                       // [4][16][pb Nwex + 1] complex
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
     // rows of a stage that no box writes only feed accumulator entries that
@@ -519,7 +599,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int col0 = part * ncp;
         const int n_l = MODE == 2 ? 0 : i % P.nb, k_l = MODE == 2 ? 0 : i / P.nb;
         const int rs = P.pb * P.Nwex + 1;      // entries of a row's buffer (odd: no bank conflicts)
-        double* buf = bufs + (size_t)quad * 16 * (kRowEnt + 1) * 2;
+        double* buf = bufs + (size_t)quad * 16 * rs * 2;
         int* eb = ebs + quad * kMaxN;
         const int pr = lane >> 1;
         // this thread's share of the quarter's stores and column exponents
@@ -553,43 +633,53 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
         };
         int t = f_tile_of(P, 0);
-        FTile x{};
         int eA = 0, eC = 0;
-        if (t < P.ntiles) {
-            x = f_tile<MODE>(P, t);
-            exps(x, eA, eC);
-        }
+        if (t < P.ntiles) exps(f_tile<MODE>(P, t), eA, eC);
         uint32_t tl = 0;
         for (int it = 0; t < P.ntiles; ++it, ++tl) {
-            // the next tile's entry and exponents are loaded while this one is drained
-            const int tn = f_tile_of(P, it + 1);
-            const FTile xn = f_tile<MODE>(P, tn < P.ntiles ? tn : t);
-            int eAn, eCn;
-            // sum of the levels in units of 2^54: level p counts 2^(42-8p)
-            long long V[16];
+            // sum of the levels, level p counting 2^(56-8p): (hi, mid, lo)
+            uint32_t lo[16], mid[16], hi[16];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) V[u] = 0;
+            for (int u = 0; u < 16; ++u) lo[u] = mid[u] = hi[u] = 0u;
             bool fail = false;
 #pragma unroll
             for (int p = 0; p < kDig; ++p) {
                 if (!fail) fail = __any_sync(0xffffffffu, !mbar_wait(&tfull[p], tl & 1, P.budget, abort_flag));
                 if (fail) continue;
                 tc_fence_after();
-                float v[16];
-                tmem_ld16(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(p * kMaxN + col0), v);
-                tmem_wait_ld();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[p]);
+                const uint32_t ta = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(p * kMaxN + col0);
 #pragma unroll
-                for (int u = 0; u < 16; ++u) {
-                    const int w = __float2int_rn(v[u]);
-                    if (p < 2) V[u] += (long long)((unsigned long long)(long long)w << (42 - 8 * p));
-                    else if (p < 6) V[u] += (long long)w * (1 << (42 - 8 * (p < 2 ? 2 : p > 5 ? 5 : p)));
-                    else V[u] += (w + 32) >> 6;
+                for (int u0 = 0; u0 < 16; u0 += 8) {   // eight at a time: registers
+                    float v[8];
+                    tmem_ld8(ta + u0, v);
+                    tmem_wait_ld();
+                    if (u0 == 8) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&tempty[p]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int u = u0 + k, w = __float2int_rn(v[k]);
+                        switch (p) {
+                            case 0: add_level<0>(lo[u], mid[u], hi[u], w); break;
+                            case 1: add_level<1>(lo[u], mid[u], hi[u], w); break;
+                            case 2: add_level<2>(lo[u], mid[u], hi[u], w); break;
+                            case 3: add_level<3>(lo[u], mid[u], hi[u], w); break;
+                            case 4: add_level<4>(lo[u], mid[u], hi[u], w); break;
+                            case 5: add_level<5>(lo[u], mid[u], hi[u], w); break;
+                            case 6: add_level<6>(lo[u], mid[u], hi[u], w); break;
+                            default: add_level<7>(lo[u], mid[u], hi[u], w);
+                        }
+                    }
                 }
             }
-            exps(xn, eAn, eCn);
+            // the tile's entry is decoded only now (registers), and the next one's
+            // exponents are loaded while this one is stored
+            const int tn = f_tile_of(P, it + 1);
+            const FTile x = f_tile<MODE>(P, t);
+            int eAn, eCn;
+            exps(f_tile<MODE>(P, tn < P.ntiles ? tn : t), eAn, eCn);
             if (tq < kMaxN) eb[tq] = eC;
             // the previous tile's stores have read the buffer
             bulk_wait_read_all();
@@ -600,8 +690,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                 double2* dst = P.scr + ((size_t)x.Ql * P.N + K1) * P.N + x.j0 + col0 + c;
 #pragma unroll
                 for (int u = 0; u < 16; u += 2) {
-                    const double v0 = fixed_to_f64(V[u], eA + eb[col0 + u] - 54, false);
-                    const double v1 = fixed_to_f64(V[u + 1], eA + eb[col0 + u + 1] - 54, false);
+                    const double v0 = fixed_to_f64(lo[u], mid[u], hi[u], eA + eb[col0 + u] - 68, false);
+                    const double v1 = fixed_to_f64(lo[u + 1], mid[u + 1], hi[u + 1], eA + eb[col0 + u + 1] - 68, false);
                     const double y = __shfl_xor_sync(0xffffffffu, c ? v0 : v1, 1);
                     if (K1 < P.N && x.j0 + col0 + u + c < P.N) dst[u] = c ? make_double2(y, v1) : make_double2(v0, y);
                 }
@@ -610,7 +700,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
                 for (int u = 0; u < 16; ++u) {
                     const uint32_t dst = (dstp[u >> 2] >> (8 * (u & 3))) & 0xFFu;
-                    const double val = fixed_to_f64(V[u], eA + eb[col0 + u] - 54, MODE == 0);
+                    const double val = fixed_to_f64(lo[u], mid[u], hi[u], eA + eb[col0 + u] - 68, MODE == 0);
                     if (dst != 255) buf[(pr * rs + dst) * 2 + c] = val;
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -647,7 +737,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                 bulk_commit();
             }
             t = tn;
-            x = xn;
             eA = eAn;
             eC = eCn;
         }
@@ -698,7 +787,7 @@ struct F64Plan {
     int* pos0 = nullptr;
     __half* X = nullptr;
     int* ex = nullptr;
-    __half* ab = nullptr;      // direct: [2][nQg * 7][N][2][Bp]
+    __half* ab = nullptr;      // direct: [2][nQg * 8][N][3][Bp]
     int* exab = nullptr;       // [2][nQg][N]
     double2* scr = nullptr;    // [nQg][N][N]
     CUtensorMap mA, mB, dA, dB;
@@ -719,8 +808,9 @@ PFN_cuTensorMapEncodeTiled_v12000 f_encoder() {
     return fn;
 }
 
-int f_smem(int ncols) {
-    return std::max(kMinSmem, kStages * kDig * (kAPlane + ncols * 64) + 1024 + 256 + 4 * kMaxN * 4 + 4 * 16 * (kRowEnt + 1) * 16);
+// Shared memory of k_gemm_digits; entries: pb Nwex of a row's run buffer (0: direct).
+int f_smem(int ncols, int entries) {
+    return kStages * kDig * (kAPlane + ncols * 64) + 1024 + 256 + 4 * kMaxN * 4 + 4 * 16 * (entries + 1) * 16;
 }
 
 bool encode_maps(const G4Dims& d, F64Plan& X) {
@@ -761,9 +851,9 @@ bool choose_tile(const G4Dims& d, int nsteps, F64Plan& X) {
         for (int kb = 1; kb <= d.Nc && 2 * kb * nb <= kARows; ++kb)
             for (int pb = 1; pb <= d.Nc; ++pb) {
                 const int N = (W * pb + 15) / 16 * 16;
-                if (N > kMaxN || pb * d.Nwex > kRowEnt) break;
+                if (N > kMaxN || f_smem(N, pb * d.Nwex) > kMaxSmem) break;
                 const int nkb = (d.Nc + kb - 1) / kb, npb = (d.Nc + pb - 1) / pb;
-                const double cost = blocks * nkb * npb * (std::max((kARows + N) / 4.0 * 28 * nsteps, 1500.0 + 90.0 * N) + 500.0);
+                const double cost = blocks * nkb * npb * (std::max((kARows + N) / 4.0 * 36 * nsteps, 1700.0 + 130.0 * N) + 500.0);
                 if (cost < best) {
                     best = cost;
                     X.kb = kb;
@@ -876,7 +966,7 @@ void f64tc_prepare(g4_ctx* h) {
     ok = ok && cudaMemset(X->ex, 0, (size_t)X->gcap * d.N * sizeof(int)) == cudaSuccess &&
          cudaMemcpy(X->work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(X->pos0, pos0.data(), pos0.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
-         encode_maps(d, *X) && raise_smem_limit(k_gemm_digits<0>) == cudaSuccess &&
+         encode_maps(d, *X) && raise_smem_limit(k_spread) == cudaSuccess && raise_smem_limit(k_gemm_digits<0>) == cudaSuccess &&
          raise_smem_limit(k_gemm_digits<1>) == cudaSuccess && raise_smem_limit(k_gemm_digits<2>) == cudaSuccess &&
          cudaDeviceGetAttribute(&X->sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess;
     if (!ok) {
@@ -884,8 +974,8 @@ void f64tc_prepare(g4_ctx* h) {
         f_free(X);
         return;
     }
-    X->smem = f_smem(X->N);
-    X->dsmem = f_smem(kMaxN);
+    X->smem = std::max(kMinSmem, f_smem(X->N, X->pb * d.Nwex));
+    X->dsmem = std::max(kMinSmem, f_smem(kMaxN, 0));
     h->bytes += held;
     h->f64tc = X;
 }
@@ -896,7 +986,8 @@ void f64tc_release(g4_ctx* h) {
 }
 
 bool f64tc_wanted(const g4_ctx* h, int staged) {
-    if (!h->f64tc || (double)h->d.E * staged < kF64tcMinUpdates) return false;
+    // fewer than four measurements: k_spread has no quarter to spare
+    if (!h->f64tc || staged < 4 || (double)h->d.E * staged < kF64tcMinUpdates) return false;
     // the sign factors must stay in the digits' exponent range
     for (int r = 0; r < staged; ++r) {
         const double a = std::fabs(h->slot_sign[r]);
@@ -908,11 +999,13 @@ bool f64tc_wanted(const g4_ctx* h, int staged) {
 g4_status f64tc_run(g4_ctx* h, int staged) {
     const F64Plan* X = (const F64Plan*)h->f64tc;
     const G4Dims& d = h->d;
-    const unsigned* flag = h->gmax;
+    unsigned* flag = h->gmax;
     FSigns sg{};
+    SpreadArgs sp{};
     for (int r = 0; r < staged; ++r) {
         sg.rs[r] = std::sqrt(std::fabs(h->slot_sign[r]));
         sg.neg[r] = h->slot_sign[r] < 0.0;
+        sp.se[r] = sg.rs[r] > 0.0 ? (signed char)std::ilogb(sg.rs[r]) : (signed char)-128;
     }
     FParams P{};
     P.acc = h->acc;
@@ -957,6 +1050,14 @@ g4_status f64tc_run(g4_ctx* h, int staged) {
     }
     const int njb = (d.Nw2 + kPackJ - 1) / kPackJ;
     cudaError_t e;
+    prof_begin(h, G4_K_PACK_EXCHANGE);
+    const bool direct = has_direct(d.ch);
+    const size_t ssm = (size_t)(direct ? 3 : 2) * staged * 256 * sizeof(unsigned short);
+    const long long sblocks = ((long long)d.N * d.N + 255) / 256;
+    k_spread<<<(int)std::min<long long>(sblocks, 16LL * X->sms), 256, ssm, h->stream>>>(h->Gfull, staged, sp, direct, d,
+                                                                                       flag);
+    prof_end(h, G4_K_PACK_EXCHANGE);
+    if ((e = cudaGetLastError()) != cudaSuccess) return g4_cuda_fail(h, e, "digit spread launch");
     for (size_t g = 0; g < X->gd0.size(); ++g) {
         prof_begin(h, G4_K_PACK_EXCHANGE);
         k_pack_digits<<<dim3(d.Nc * njb, d.N), 256, kPackJ * 2 * (X->J + 2) * sizeof(double), h->stream>>>(
@@ -977,7 +1078,7 @@ g4_status f64tc_run(g4_ctx* h, int staged) {
         prof_end(h, G4_K_EXCHANGE);
         if ((e = cudaGetLastError()) != cudaSuccess) return g4_cuda_fail(h, e, "digit exchange launch");
     }
-    if (!has_direct(d.ch)) return G4_OK;
+    if (!direct) return G4_OK;
     P.scr = X->scr;
     P.exA = X->exab;
     P.exB = X->exab + (size_t)X->nQg * d.N;
