@@ -86,9 +86,11 @@ typedef enum {
                               of one spin lie more than 2^7 below the entry's largest
                               value, or are outside 2^+-380, takes the plain kernels
                               (the digits' error is relative to the largest value).  The
-                              tensor-core form keeps up to an eighth of the device memory
-                              free at g4_create, at most 8 GB, for its operands and is
-                              not used with mem_limit or timeout_cycles */
+                              tensor-core form keeps as much device memory for its
+                              operands as the accumulator and the staged G take (at least
+                              512 MB, at most 4 GB, never more than the problem needs); it
+                              is not used with mem_limit or timeout_cycles, nor where that
+                              memory cannot be had */
     G4_PREC_MIXED = 1      /* batched path: complex64 G, exchange-type term on tensor
                               cores (3-term FP16 or TF32 split, FP32 accumulate) or FP32
                               CUDA cores, added to the FP64 accumulator once per batch;
@@ -296,7 +298,10 @@ g4_status g4_reset(g4_handle h);
  * pending operands and scale, the kept exchange operand scale of deferred
  * staging, sign sum, measurement count, problem description) to / from a
  * file.  Staged measurements are accumulated first.  A restored run
- * continues exactly (bit for bit) as the interrupted one would have.
+ * continues exactly (bit for bit) as the interrupted one would have: an FP64
+ * run with the kernels it was begun with (plain or tensor-core form; only where
+ * the latter has no memory, or the handle mem_limit or timeout_cycles, does it go
+ * on with the plain ones, to rounding).
  * Restoring into a handle of a different problem, or one whose direct-term
  * window is smaller than the saved fill, gives G4_ERR_INVALID.  Both calls
  * synchronise the handle's stream.

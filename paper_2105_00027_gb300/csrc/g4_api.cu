@@ -429,6 +429,7 @@ g4_status g4_reset(g4_handle h) {
     G4_CUDA(h, cudaMemsetAsync(h->dstatus, 0, kStatusWords * sizeof(unsigned), h->stream));
     direct_reset(h);
     h->scaled = false;
+    h->f64_plain = false;
     h->staged = 0;
     h->sign_sum = 0.0;
     h->nmeas = 0;
@@ -671,7 +672,10 @@ struct CkptHeader {
     int accum;
     unsigned gscale;   // the kept exchange operand scale (deferred staging), so that a
                        // restored run continues bit for bit
+    int fp64_form;     // FP64 handles: 1 plain kernels alone, 2 tensor-core form; other
+                       // values (files written before this field): not recorded
 };
+static_assert(sizeof(CkptHeader) == 88, "the file format has no other fields");
 constexpr size_t kIoChunk = (size_t)256 << 20;
 }  // namespace
 
@@ -715,6 +719,7 @@ g4_status g4_checkpoint(g4_handle h, const char* path) {
     hd.window_max = wmax;
     hd.accum = h->opt.accum;
     hd.gscale = gscale;
+    hd.fp64_form = h->f64tc && !h->f64_plain ? 2 : 1;
     FILE* f = std::fopen(path, "wb");
     if (!f) return g4_fail(h, G4_ERR_INVALID, std::string("cannot open ") + path);
     bool ok = std::fwrite(&hd, sizeof(hd), 1, f) == 1;
@@ -784,6 +789,12 @@ g4_status g4_restore(g4_handle h, const char* path) {
     if (st != G4_OK) return st;
     G4_CUDA(h, cudaMemcpy(h->gscale, &hd.gscale, sizeof(unsigned), cudaMemcpyHostToDevice));
     h->scaled = true;
+    // the run goes on with the kernels it was begun with, whatever memory was
+    // free when this handle was made
+    if (h->opt.precision == G4_PREC_FP64) {
+        h->f64_plain = hd.fp64_form == 1;
+        if (hd.fp64_form == 2 && !h->f64tc) f64tc_prepare(h);
+    }
     h->sign_sum = hd.sign_sum;
     h->nmeas = hd.nmeas;
     h->staged = 0;

@@ -229,22 +229,37 @@ __global__ void __launch_bounds__(256) k_spread(const double2* __restrict__ G, i
 // A block takes one row i and eight consecutive columns j of one momentum: it
 // reads one 128-byte line of every slot and spin, and writes whole rows of X
 // (2 J bytes per digit and component).  Values r >= staged are zero, written
-// up to the next multiple of 32 (the GEMM's chunks of K).  HBM-bound: 16 B
+// up to the next multiple of 32 (the GEMM's chunks of K).  The group's diagonals
+// have dn0 <= |dn| <= dn1, so that a row meets them in two bands of columns:
+// blockIdx.x / Nc counts band 0's nband blocks, then band 1's (a launch over all
+// columns, left at once by the blocks without one of the group, took 0.28 ms a
+// group on the 4x4 cluster with 64 frequencies).  HBM-bound: 16 B
 // read and 48 B written per entry, slot and spin.
 constexpr int kPackJ = 8;
 
 __global__ void __launch_bounds__(256) k_pack_digits(const double2* __restrict__ G, int staged, int Jh,
                                                      int live, FSigns sg, const int* __restrict__ pos0,
-                                                     int a0, int na, __half* __restrict__ X,
+                                                     int a0, int na, int dn0, int dn1, int nband,
+                                                     __half* __restrict__ X,
                                                      int* __restrict__ ex, G4Dims d,
                                                      const unsigned* __restrict__ flag) {
     if (*flag) return;
     extern __shared__ __align__(16) double xs[];   // [kPackJ][2][ld]
     const int J = 2 * Jh, ld = J + 2;
-    const int njb = (d.Nw2 + kPackJ - 1) / kPackJ;
-    const int k = blockIdx.x / njb, n0 = (blockIdx.x - k * njb) * kPackJ;
     const int i = blockIdx.y, kr = i / d.Nw2, ni = i - kr * d.Nw2;
-    const int nv = min(kPackJ, d.Nw2 - n0);
+    const int bx = blockIdx.x / d.Nc, k = blockIdx.x - bx * d.Nc;
+    // column blocks of n = ni - dn1 .. ni - dn0, then those of ni + dn0 .. ni + dn1
+    // that the first band does not have
+    const int end0 = ni - dn0 >= 0 ? (ni - dn0) / kPackJ + 1 : 0;
+    int jb;
+    if (bx < nband) {
+        jb = max(0, ni - dn1) / kPackJ + bx;
+        if (jb >= end0) return;
+    } else {
+        jb = max((ni + dn0) / kPackJ, end0) + bx - nband;
+        if (jb * kPackJ > min(d.Nw2 - 1, ni + dn1)) return;
+    }
+    const int n0 = jb * kPackJ, nv = min(kPackJ, d.Nw2 - n0);
     int dkx = kr % d.Lx - k % d.Lx, dky = kr / d.Lx - k / d.Lx;
     dkx += dkx < 0 ? d.Lx : 0;
     dky += dky < 0 ? d.Ly : 0;
@@ -876,16 +891,21 @@ void f_free(F64Plan* X) {
     delete X;
 }
 
-// Device memory the plan may take: an eighth of what is free when the handle
-// is made, at most 8 GB (the operands of a batch are formed in groups of
-// diagonals that fit).
-constexpr size_t kMaxPlanBytes = (size_t)8 << 30;
+// Device memory the plan may take (the operands of a batch are formed in groups
+// of diagonals that fit): by the problem's sizes alone, as much as the
+// accumulator and the staged G take, at least 512 MB and at most 4 GB.  One batch
+// of 64 on the 4x4 cluster with 64 frequencies and 8 x 16 transfers takes 20.7
+// ms with 4 GB (four groups), 20.1 with 8 (two), 21.4 with 2, 22.4 with 1.
+size_t plan_bytes(const G4Dims& d, int batch) {
+    const size_t held = ((size_t)d.E + (size_t)batch * 2 * d.N * d.N) * sizeof(double2);
+    return std::min<size_t>(std::max<size_t>(held, (size_t)512 << 20), (size_t)4 << 30);
+}
 
 }  // namespace
 
 void f64tc_prepare(g4_ctx* h) {
     const G4Dims& d = h->d;
-    // below 2^18 element-updates a batch is a few microseconds of the plain
+    // below kF64tcMinUpdates element-updates a batch is some 0.1 ms of the plain
     // kernel; a memory limit or a wait budget of the caller's is kept as it was
     if (h->opt.mem_limit > 0 || h->opt.timeout_cycles > 0) return;
     if (d.Nwex > kMaxWex || (double)d.E * h->batch < kF64tcMinUpdates) return;
@@ -897,19 +917,19 @@ void f64tc_prepare(g4_ctx* h) {
     if (X->Jh > 16) X->Jh = (X->Jh + 31) / 32 * 32;
     X->J = 2 * X->Jh;
     X->Bp = (h->batch + 31) / 32 * 32;
-    size_t free_b = 0, total_b = 0;
     std::vector<int2> dl;
     std::vector<int> itemlen;
     diag_list(d, dl, itemlen);
-    bool ok = choose_tile(d, X->J / 8, *X) && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess;
-    const size_t budget = std::min(kMaxPlanBytes, free_b / 8);
+    bool ok = choose_tile(d, X->J / 8, *X);
+    const size_t budget = plan_bytes(d, h->batch);
     // direct term: transfers per group, whose scratch stays in L2 where it can
     size_t direct_b = 0;
     if (has_direct(d.ch)) {
         const size_t one = (size_t)d.N * d.N * sizeof(double2);
         X->nQg = (int)std::min<size_t>(std::min(kGroupQ, d.NQ), std::max<size_t>(4, ((size_t)64 << 20) / one));
-        X->nQg = std::min(X->nQg, d.NQ);
-        direct_b = X->nQg * (one + (size_t)2 * d.N * (3 * X->Bp * kDig * sizeof(__half) + sizeof(int)));
+        const size_t per_Q = one + (size_t)2 * d.N * (3 * X->Bp * kDig * sizeof(__half) + sizeof(int));
+        X->nQg = (int)std::min<size_t>(std::min(X->nQg, d.NQ), std::max<size_t>(1, budget / 2 / per_Q));
+        direct_b = X->nQg * per_Q;
     }
     const size_t per_diag = (size_t)d.N * (3 * X->J * kDig * sizeof(__half) + sizeof(int));
     ok = ok && budget > direct_b && (budget - direct_b) / per_diag >= 2;
@@ -987,7 +1007,7 @@ void f64tc_release(g4_ctx* h) {
 
 bool f64tc_wanted(const g4_ctx* h, int staged) {
     // fewer than four measurements: k_spread has no quarter to spare
-    if (!h->f64tc || staged < 4 || (double)h->d.E * staged < kF64tcMinUpdates) return false;
+    if (!h->f64tc || h->f64_plain || staged < 4 || (double)h->d.E * staged < kF64tcMinUpdates) return false;
     // the sign factors must stay in the digits' exponent range
     for (int r = 0; r < staged; ++r) {
         const double a = std::fabs(h->slot_sign[r]);
@@ -1060,8 +1080,12 @@ g4_status f64tc_run(g4_ctx* h, int staged) {
     if ((e = cudaGetLastError()) != cudaSuccess) return g4_cuda_fail(h, e, "digit spread launch");
     for (size_t g = 0; g < X->gd0.size(); ++g) {
         prof_begin(h, G4_K_PACK_EXCHANGE);
-        k_pack_digits<<<dim3(d.Nc * njb, d.N), 256, kPackJ * 2 * (X->J + 2) * sizeof(double), h->stream>>>(
-            h->Gfull, staged, X->Jh, live, sg, X->pos0, X->gd0[g], X->gdn[g], X->X, X->ex, d, flag);
+        // |dn| of the group's first and last diagonal (see diag_pos)
+        auto dn_of = [&](int pos) { return pos < d.Nc ? 0 : (pos - d.Nc) / (2 * d.Nc) + 1; };
+        const int dn0 = dn_of(X->gd0[g]), dn1 = dn_of(X->gd0[g] + X->gdn[g] - 1);
+        const int nband = std::min(njb, (dn1 - dn0) / kPackJ + 2);
+        k_pack_digits<<<dim3(d.Nc * 2 * nband, d.N), 256, kPackJ * 2 * (X->J + 2) * sizeof(double), h->stream>>>(
+            h->Gfull, staged, X->Jh, live, sg, X->pos0, X->gd0[g], X->gdn[g], dn0, dn1, nband, X->X, X->ex, d, flag);
         prof_end(h, G4_K_PACK_EXCHANGE);
         if ((e = cudaGetLastError()) != cudaSuccess) return g4_cuda_fail(h, e, "digit pack launch");
         P.work = X->work + X->gw0[g];

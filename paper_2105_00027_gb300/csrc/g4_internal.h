@@ -131,6 +131,8 @@ struct g4_ctx {
     void* f64tc = nullptr;           // batch update on tensor cores (g4_fp64_tc.cu), or null;
                                      // *gmax is then the batch's flag: a G entry that only
                                      // the plain kernels take
+    bool f64_plain = false;          // this run (restored) started on a handle without f64tc: plain
+                                     // kernels until the next reset
 
     // mixed path
     float2* Gd = nullptr;            // [batch*2][Nc dk][ndn][Nc k][Nw2 n] complex64,
