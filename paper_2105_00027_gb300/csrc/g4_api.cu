@@ -21,7 +21,7 @@ std::atomic<unsigned long long> g_next_uid{1};
 
 // Executable graphs of g4_accumulate_group, one per group signature: the
 // handles (by identifier) in launch order, the number of measurements each had
-// staged, whether its accumulator was still to be written and how full its direct-term window was (which decides where the
+// staged and how full its direct-term window was (which decides where the
 // batch's operands go and whether the window is added).  While a group's
 // batches keep that shape the graph is relaunched as it is, and each handle's
 // window then advances as it did when the graph was captured; a destroyed
@@ -29,9 +29,8 @@ std::atomic<unsigned long long> g_next_uid{1};
 struct GroupKey {
     unsigned long long uid;
     int staged, fill;
-    bool fresh;   // the batch writes the accumulator instead of adding to it
     bool operator==(const GroupKey& o) const {
-        return uid == o.uid && staged == o.staged && fill == o.fill && fresh == o.fresh;
+        return uid == o.uid && staged == o.staged && fill == o.fill;
     }
 };
 struct GroupGraph {
@@ -165,7 +164,8 @@ g4_status accumulate_mixed(g4_ctx* h) {
 // Clear an accumulator that no batch has written.
 g4_status clear_fresh(g4_ctx* h) {
     if (!h->fresh) return G4_OK;
-    G4_CUDA(h, cudaMemsetAsync(h->acc, 0, (size_t)h->d.E * sizeof(double2), h->stream));
+    G4_CUDA(h, launch_clear_unset(h->acc, h->accset, h->d, h->stream));
+    G4_CUDA(h, cudaMemsetAsync(h->accset, 1, sizeof(unsigned), h->stream));
     h->fresh = false;
     return G4_OK;
 }
@@ -357,6 +357,13 @@ g4_status g4_create(int Nc, int Nw, int Nwex, int Nkex, g4_channel ch, const g4_
     h->gmax = h->dstatus + 1;
     h->gscale = h->dstatus + 2;
     h->gredo = h->dstatus + 3;
+    h->accset = h->dstatus + 4;
+    // (until the reset below: the tuning runs add, as a run's batches do)
+    ce = cudaMemset(h->accset, 1, sizeof(unsigned));
+    if (ce != cudaSuccess) {
+        g4_cuda_fail(h, ce, "status words");
+        return fail(G4_ERR_CUDA);
+    }
     ce = cudaHostAlloc((void**)&h->hstatus, sizeof(unsigned), cudaHostAllocDefault);
     if (ce != cudaSuccess) {
         g4_cuda_fail(h, ce, "cudaHostAlloc");
@@ -421,12 +428,12 @@ g4_status g4_create(int Nc, int Nw, int Nwex, int Nkex, g4_channel ch, const g4_
 
 g4_status g4_reset(g4_handle h) {
     if (!h) return G4_ERR_INVALID;
-    h->fresh = true;
-    if (!h->xtc || h->opt.accum == G4_ACCUM_F32PAIR) {
-        g4_status st = clear_fresh(h);
-        if (st != G4_OK) return st;
-    }
     G4_CUDA(h, cudaMemsetAsync(h->dstatus, 0, kStatusWords * sizeof(unsigned), h->stream));
+    h->fresh = h->xtc && h->opt.accum != G4_ACCUM_F32PAIR;
+    if (h->fresh)
+        G4_CUDA(h, launch_clear_diag(h->acc, h->d, h->stream));
+    else
+        G4_CUDA(h, cudaMemsetAsync(h->acc, 0, (size_t)h->d.E * sizeof(double2), h->stream));
     direct_reset(h);
     h->scaled = false;
     h->f64_plain = false;
@@ -508,14 +515,17 @@ g4_status g4_accumulate_group(g4_handle* hs, int n) {
     const cudaStream_t main = h0->stream;  // may be the legacy stream, which cannot capture
     const int nb = (int)work.size();
     std::vector<GroupKey> key;
-    for (g4_ctx* h : work) key.push_back(GroupKey{h->uid, h->staged, direct_fill(h), h->fresh});
+    for (g4_ctx* h : work) key.push_back(GroupKey{h->uid, h->staged, direct_fill(h)});
     {
         // a group shape seen before: relaunch its graph
         std::lock_guard<std::mutex> lock(g_graph_mu);
         for (const GroupGraph& gg : g_graphs)
             if (gg.key == key) {
                 cudaError_t e = cudaGraphLaunch(gg.exec, main);
-                if (e != cudaSuccess) return g4_cuda_fail(h0, e, "grouped accumulate graph launch");
+                if (e != cudaSuccess) {
+                    cudaGetLastError();
+                    return g4_cuda_fail(h0, e, "grouped accumulate graph launch");
+                }
                 for (size_t i = 0; i < work.size(); ++i) {
                     work[i]->staged = 0;
                     work[i]->fresh = false;
@@ -573,6 +583,14 @@ g4_status g4_accumulate_group(g4_handle* hs, int n) {
         gg.exec = exec;
         g_graphs.push_back(gg);
         exec = nullptr;
+        for (g4_ctx* h : work) h->fresh = false;
+    } else {
+        // nothing has run: what the capture changed on the host is put back
+        for (int i = 0; i < nb; ++i) {
+            work[i]->staged = key[i].staged;
+            direct_set_fill(work[i], key[i].fill);
+        }
+        cudaGetLastError();   // reported below, not by the next launch
     }
     // streams, events and the graph description are released once their work completes
     if (exec) cudaGraphExecDestroy(exec);

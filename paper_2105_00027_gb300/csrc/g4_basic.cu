@@ -492,6 +492,21 @@ __global__ void __launch_bounds__(256) k_build_G_diag(const void* __restrict__ M
     if (threadIdx.x == 0) atomicMax(gmax, bmax);
 }
 
+// Zero the accumulator's entries with K1 = K2 (the diagonal D = 0, whose split
+// tiles in the tensor-core exchange add their partial sums also in the first
+// batch).
+__global__ void k_clear_diag(double2* __restrict__ acc, int N, int NQ) {
+    double2* row = acc + ((size_t)blockIdx.x * N + blockIdx.x) * NQ;
+    for (int i = threadIdx.x; i < NQ; i += blockDim.x) row[i] = make_double2(0.0, 0.0);
+}
+
+__global__ void k_clear_unset(double2* __restrict__ acc, long long E, const unsigned* __restrict__ accset) {
+    if (*accset) return;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < E;
+         i += (long long)gridDim.x * blockDim.x)
+        acc[i] = make_double2(0.0, 0.0);
+}
+
 constexpr long long kTiledMinEntries = 1 << 18;
 
 }  // namespace
@@ -581,6 +596,16 @@ cudaError_t launch_finalize(const double2* acc, bool pair, double inv_s, double2
     auto* k = pair ? k_finalize<true, false> : scr ? k_finalize<false, true> : k_finalize<false, false>;
     k<<<grid, kFinThreads, RC * per, s>>>(acc, scr, scr0, inv_s, out, d, TQ, RC, nsplit, n2_0, n2_cnt, q0, nq,
                                           out_plane);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_clear_diag(double2* acc, const G4Dims& d, cudaStream_t s) {
+    k_clear_diag<<<d.N, 128, 0, s>>>(acc, d.N, d.NQ);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_clear_unset(double2* acc, const unsigned* accset, const G4Dims& d, cudaStream_t s) {
+    k_clear_unset<<<(int)std::min<long long>((d.E + 255) / 256, 152 * 16), 256, 0, s>>>(acc, d.E, accset);
     return cudaGetLastError();
 }
 

@@ -711,13 +711,6 @@ __global__ void __launch_bounds__(256) k_max_M(const __grid_constant__ G4SlotTab
     if (threadIdx.x == 0) atomicMax(gscale, bmax);
 }
 
-// Zero the accumulator's entries with K1 = K2 (the diagonal D = 0, whose split
-// tiles add their partial sums also in the first batch).
-__global__ void k_clear_diag(double2* __restrict__ acc, int N, int NQ) {
-    double2* row = acc + ((size_t)blockIdx.x * N + blockIdx.x) * NQ;
-    for (int i = threadIdx.x; i < NQ; i += blockDim.x) row[i] = make_double2(0.0, 0.0);
-}
-
 // ---------------------------------------------------------------- tensor-core kernel
 struct TParams {
     double2* acc;
@@ -737,7 +730,8 @@ struct TParams {
     uint32_t idesc;
     const unsigned* gmax;  // FP16 operands: largest |G~| component of the batch (FP32 bits)
     int pair;              // accumulator of compensated FP32 pairs (else FP64)
-    int store;             // the accumulator's first batch: runs are written, not added
+    const unsigned* accset;  // *accset == 0: the accumulator's first batch, runs are written,
+                             // not added (null: always added)
     long long budget;
 };
 
@@ -1066,6 +1060,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int rs = run_stride(P.Nwex);
         double2* runs = (double2*)(smem + kStages * stage_bytes + 256) + (size_t)ew * kRunBufs * 16 * rs;
         const int pr = lane >> 1;              // row pair of this lane within the warp
+        const bool store = P.accset && *P.accset == 0u;
         uint32_t tl = 0, wb = 0;
         bool live = true;
         for (int it = 0; live; ++it) {
@@ -1153,7 +1148,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (c == 0) {
-                        if (P.store && !x.split) {
+                        if (store && !x.split) {
                             // the first batch writes every entry of its rows, the structurally
                             // zero ones too: no clear before, and no read here
                             if (nh == 2 && qv[1] < P.Nkex && qv[1] == qv[0] + 1) {
@@ -1574,8 +1569,8 @@ g4_status xtc_prepare(g4_ctx* h) {
     // The tile shape: the cost model's choice, or -- with autotuning on and no
     // short wait budget -- the fastest of its best few candidates, each timed
     // over one full batch on the handle's own buffers (the staged G is still
-    // all zero, so the accumulator, cleared when the handle is made, is left
-    // unchanged), best of two after a warm-up.
+    // all zero; the accumulator's contents mean nothing before the reset that ends
+    // g4_create), best of two after a warm-up.
     Tile best = cands[0];
     const bool tune = h->opt.autotune && h->opt.timeout_cycles == 0 && cands.size() > 1;
     if (tune) {
@@ -1660,17 +1655,12 @@ g4_status xtc_run(g4_ctx* h, int staged) {
     P.pair = h->opt.accum == G4_ACCUM_F32PAIR;
     // The first batch after a reset writes the accumulator, which is then neither
     // cleared before nor read: every entry off the diagonal D = 0 belongs to one
-    // tile.
+    // tile.  *accset is set behind the batch's last launch, so that a batch whose
+    // launches failed is not taken for one that has written.
     // Measured per run, clear and first batch's read saved: 8x8 cluster, 32
     // frequencies, two batches 43.6 -> 41.7 ms; 6x6, two batches 40.2 -> 39.1;
     // 4x4, one batch from vertices 7.49 -> 7.21.
-    P.store = h->fresh;
-    if (h->fresh) {
-        k_clear_diag<<<d.N, 128, 0, h->stream>>>(h->acc, d.N, d.NQ);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return g4_cuda_fail(h, e, "accumulator diagonal clear");
-        h->fresh = false;
-    }
+    P.accset = P.pair ? nullptr : h->accset;
     P.budget = h->opt.timeout_cycles > 0 ? h->opt.timeout_cycles : 4000000000LL;
     // deferred staging: the G0 all staged measurements share, if they do
     const double2* g0s = nullptr;
@@ -1758,6 +1748,15 @@ g4_status xtc_run(g4_ctx* h, int staged) {
                 if (e != cudaSuccess) return g4_cuda_fail(h, e, "tensor-core exchange launch");
             }
         }
+    }
+    // under capture nothing has run yet, and the launches may follow any reset
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) cudaGetLastError();
+    const bool captured = cap == cudaStreamCaptureStatusActive;
+    if (P.accset && (h->fresh || captured)) {
+        cudaError_t e = cudaMemsetAsync(h->accset, 1, sizeof(unsigned), h->stream);
+        if (e != cudaSuccess) return g4_cuda_fail(h, e, "accumulator flag");
+        if (!captured) h->fresh = false;
     }
     return G4_OK;
 }

@@ -48,7 +48,7 @@ inline bool has_direct(int ch) { return ch == G4_PH_MAGNETIC || ch == G4_PH_DENS
 
 // Device words of a handle: the status word, then (mixed path) the batch's
 // largest |G~| component, the kept operand scale and the pack's redo flag.
-constexpr int kStatusWords = 4;
+constexpr int kStatusWords = 5;
 
 // Device status word bits (written by kernels whose bounded waits give up).
 enum : unsigned { G4_DEV_TIMEOUT = 1u, G4_DEV_BADARG = 2u };
@@ -116,8 +116,13 @@ struct g4_ctx {
     // measurement (the mixed path adds the direct term once per window of
     // batches, see g4_direct_tc.cu); the exported result is acc / sum_r s_r
     double2* acc = nullptr;
-    bool fresh = false;              // acc is not cleared yet: the next batch of the tensor-core
-                                     // exchange writes it (any other use clears it first)
+    // A reset does not clear acc where the tensor-core exchange adds to it in
+    // FP64 (only the diagonal K1 = K2, see launch_clear_diag): the next batch
+    // writes it, any other use clears it first.  Which of the two a batch does is
+    // read on the device from *accset (0: not written since the reset), so that
+    // it holds for captured launches too, whenever they run.
+    unsigned* accset = nullptr;      // after dstatus
+    bool fresh = false;              // *accset may be 0
     unsigned* dstatus = nullptr;     // device status word
     unsigned* gmax = nullptr;        // largest |G~| component of the staged batch (FP32 bits),
                                      // for the FP16 operand scale; right after dstatus
@@ -212,6 +217,9 @@ void f64tc_release(g4_ctx* h);
 cudaError_t launch_finalize(const double2* acc, bool pair, double inv_s, double2* out,
                             const G4Dims& d, int n2_0, int n2_cnt, long long out_plane, int q0,
                             int nq, const float2* scr, const double2* scr0, cudaStream_t s);
+// the entries with K1 = K2 cleared; the whole accumulator, unless *accset is set
+cudaError_t launch_clear_diag(double2* acc, const G4Dims& d, cudaStream_t s);
+cudaError_t launch_clear_unset(double2* acc, const unsigned* accset, const G4Dims& d, cudaStream_t s);
 // one measurement's G~ into its batch slot of Gd, its largest component
 // joining *gmax
 cudaError_t launch_build_G_diag(const void* M, bool m64, const double2* G0, double sign,
