@@ -262,8 +262,9 @@ g4_status g4_reserve_vertices(g4_handle h, int n_max);
  * empty the batch.  No-op when nothing is staged.  On a mixed handle the
  * exchange-type term goes into the FP64 accumulator now; the direct term's
  * operands join the handle's window (options.direct_batches), whose GEMM is
- * added before a batch that does not fit and at g4_finalize (g4_checkpoint
- * saves the window with the accumulator).
+ * added before the next batch once another whole batch does not fit, and at
+ * g4_finalize (g4_checkpoint saves a window that is not full with the
+ * accumulator).
  * Errors: G4_ERR_STATE (after g4_finalize), G4_ERR_CUDA, G4_ERR_TIMEOUT.
  */
 g4_status g4_accumulate(g4_handle h);

@@ -146,15 +146,19 @@ g4_status exchange_term(g4_ctx* h) {
     return st;
 }
 
+// Whether the direct term's window is full: the next batch, if it is a whole
+// one, would not fit.
+bool window_full(const g4_ctx* h) { return direct_fill(h) + h->batch > direct_window(h); }
+
 // The exchange-type term goes into the accumulator every batch; the direct
-// term's operands join the window, whose GEMM is added before a batch that
-// would not fit (the last window's at g4_finalize).  On a deferred handle the
+// term's operands join the window, whose GEMM is added before the next batch
+// once it is full (the last window's at g4_finalize).  On a deferred handle the
 // exchange pack writes the direct operands at the window's fill, and the window
 // then takes the batch.
 g4_status accumulate_mixed(g4_ctx* h) {
     if (!has_direct(h->d.ch)) return exchange_term(h);
     g4_status st = G4_OK;
-    if (direct_fill(h) + h->staged > direct_window(h)) st = direct_flush(h);
+    if (window_full(h)) st = direct_flush(h);
     if (st == G4_OK && h->deferred) st = exchange_term(h);
     if (st == G4_OK) st = direct_pack(h, h->staged);
     if (st == G4_OK && !h->deferred) st = exchange_term(h);
@@ -702,7 +706,9 @@ g4_status g4_checkpoint(g4_handle h, const char* path) {
     g4_status st = do_accumulate(h);
     if (st == G4_OK) st = clear_fresh(h);
     if (st != G4_OK) return st;
-    if (h->finalized && (st = direct_flush(h)) != G4_OK) return st;
+    // a full window is added now, as the next batch would do: the file then goes
+    // into handles with smaller windows
+    if ((h->finalized || window_full(h)) && (st = direct_flush(h)) != G4_OK) return st;
     if ((st = sync_and_check(h)) != G4_OK) return st;
     const size_t one = (size_t)h->d.E * sizeof(double2);
     const int fill = direct_fill(h);
