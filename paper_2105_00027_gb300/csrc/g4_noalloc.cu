@@ -73,8 +73,16 @@ __global__ void k_na_build(const double2* __restrict__ M, const double2* __restr
 // 110).  The contribution is summed before it meets the accumulator: with the
 // accumulator inside the chain of fused multiply-adds, two operations fewer
 // (95 us), the error against 64 bits grew by half.
+//
+// Where the (n1, q) groups and n2 are too few blocks to fill the GPU, the
+// transfer steps (blockIdx.z % nm) and then the pairs (blockIdx.z / nm) are
+// dealt to several; each forms its own a and b.  Ten calls, one thread per entry
+// / groups alone / dealt: 16x8 cluster, N = 256, one transfer: 0.16 / 1.17 /
+// 0.16 ms; 8x8, 4 frequencies, 4 transfers: 0.24 / 0.80 / 0.22; 1x1, 128
+// frequencies, 64 transfers: 0.60 / 0.85 / 0.46.
 constexpr int kNaM = 4;
 constexpr int kNaThreads = 256;
+constexpr int kNaBlocks = 152 * 8;   // blocks that fill the GPU
 
 __device__ __forceinline__ void na_cfma(double2& t, double2 a, double2 b) {
     t.x = fma(a.x, b.x, t.x);
@@ -85,7 +93,7 @@ __device__ __forceinline__ void na_cfma(double2& t, double2 a, double2 b) {
 
 __global__ void __launch_bounds__(kNaThreads) k_na_update(const double2* __restrict__ G, double sign,
                                                           double2* __restrict__ acc, int Nc, int Lx,
-                                                          int Nw2, int Nwex, int Nkex, int gp) {
+                                                          int Nw2, int Nwex, int Nkex, int gp, int nm) {
     __shared__ double2 sa[kNaM * kNaThreads], sb[kNaM * kNaThreads];   // [m][group][k]
     const int N = Nc * Nw2, Ly = Nc / Lx, N2 = Nc * Nc;
     const size_t NN = (size_t)N * N;
@@ -97,7 +105,8 @@ __global__ void __launch_bounds__(kNaThreads) k_na_update(const double2* __restr
         y -= y >= Ly ? Ly : 0;
         return x + Lx * y;
     };
-    for (int m0 = 0; m0 < Nwex; m0 += kNaM) {
+    const int zm = blockIdx.z % nm, zp = blockIdx.z / nm, np = gridDim.z / nm;
+    for (int m0 = zm * kNaM; m0 < Nwex; m0 += nm * kNaM) {
         __syncthreads();
         for (int t = threadIdx.x; t < ng * Nc; t += blockDim.x) {
             const int g = t / Nc, k = t - g * Nc;
@@ -122,7 +131,7 @@ __global__ void __launch_bounds__(kNaThreads) k_na_update(const double2* __restr
             }
         }
         __syncthreads();
-        for (int t = threadIdx.x; t < ng * N2; t += blockDim.x) {
+        for (int t = zp * blockDim.x + threadIdx.x; t < ng * N2; t += np * blockDim.x) {
             const int g = t / N2, r = t - g * N2, k2 = r / Nc, k1 = r - k2 * Nc;
             const int n1 = (g0 + g) / Nkex, q = (g0 + g) - n1 * Nkex;
             const int lim = min(Nwex, Nw2 - max(n1, n2)) - m0;   // transfers on the grid
@@ -241,8 +250,12 @@ extern "C" g4_status g4_update_noalloc(int Nc, int lx, int Nw, int Nwex, int Nke
     if (e != cudaSuccess) return na_fail(G4_ERR_CUDA, std::string("build launch: ") + cudaGetErrorString(e));
     // (n1, q) groups per block: as many whole Nc x Nc planes as its threads hold
     const int gp = std::max(1, kNaThreads / (Nc * Nc)), groups = 2 * Nw * Nkex;
-    k_na_update<<<dim3((groups + gp - 1) / gp, 2 * Nw), kNaThreads, 0, s>>>(G, sign, (double2*)acc, Nc, Lx, 2 * Nw,
-                                                                            Nwex, Nkex, gp);
+    const int bx = (groups + gp - 1) / gp, blocks2 = bx * 2 * Nw;
+    const int nm = std::min((Nwex + kNaM - 1) / kNaM, (kNaBlocks + blocks2 - 1) / blocks2);
+    const int np = std::min((std::min(gp, groups) * Nc * Nc + kNaThreads - 1) / kNaThreads,
+                            (kNaBlocks + blocks2 * nm - 1) / (blocks2 * nm));
+    k_na_update<<<dim3(bx, 2 * Nw, nm * np), kNaThreads, 0, s>>>(G, sign, (double2*)acc, Nc, Lx, 2 * Nw, Nwex, Nkex,
+                                                                 gp, nm);
     e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(G4_ERR_CUDA, std::string("update launch: ") + cudaGetErrorString(e));
     return G4_OK;
