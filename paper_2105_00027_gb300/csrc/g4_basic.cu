@@ -311,6 +311,7 @@ constexpr int kFinNJ = 8;
 constexpr int kFinBytes = 18 * 1024;
 constexpr int kFinThreads = 128;
 constexpr long long kFinBlocks = 12288;
+constexpr int kFinWideBytes = 24 * 1024, kFinWideMax = 96 * 1024;
 
 template <bool PAIR, bool DIRECT>
 __global__ void __launch_bounds__(kFinThreads) k_finalize(
@@ -338,7 +339,7 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(
     const size_t s1 = (size_t)Nw2 * d.N, sofs = (size_t)n1 * d.N + n2;
     const float2* sp = DIRECT ? scr + (size_t)Ql * d.N * d.N + sofs : nullptr;
     const int dk2 = G / Nc, dk1 = G - dk2 * Nc;      // r += G
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
     for (int r0 = split * RC; r0 < NR; r0 += nsplit * RC) {
         const int rc = min(RC, NR - r0);
         if (mine) {
@@ -380,16 +381,58 @@ __global__ void __launch_bounds__(kFinThreads) k_finalize(
             }
         }
         __syncthreads();
-        // a warp writes one (n2, q, m) plane's run of rc entries at a time
-        for (int pl = warp; pl < nn * NJ; pl += kFinThreads / 32) {
+        // a warp writes one (n2, q, m) plane's run of rc entries at a time, or
+        // several planes' runs when they are shorter than a warp
+        const int run = rc > 16 ? 32 : rc > 8 ? 16 : rc > 4 ? 8 : rc > 2 ? 4 : rc;
+        const int pw = 32 / run, lane = (threadIdx.x & 31) % run;
+        for (int pl = warp * pw + (threadIdx.x & 31) / run; pl < nn * NJ; pl += kFinThreads / 32 * pw) {
             const int nl = pl / NJ, jj = pl - nl * NJ, qi = jj / Nwex, ml = jj - qi * Nwex;
             double2* o = out + (size_t)ml * out_plane +
                          (((size_t)(n2b + nl) * Nw2 + n1) * d.Nkex + q0 + qb + qi) * NR + r0;
             const double2* t = tileF + (size_t)nl * RC * ld + jj;
-            for (int rr = lane; rr < rc; rr += 32) {
+            for (int rr = lane; rr < rc; rr += run) {
                 const double2 v = t[(size_t)rr * ld];
                 o[rr] = make_double2(v.x * inv_s, v.y * inv_s);
             }
+        }
+        __syncthreads();
+    }
+}
+
+// The export of many transfer frequencies: a block owns one (n1, n2, q) triple,
+// 256 threads, and walks k2 in chunks of KC through shared memory, so that it
+// reads runs of Nwex contiguous entries and writes runs of KC Nc.  For more than
+// 12 transfers, on clusters of less than twelve sites for more than 8 (runs of
+// a few dozen entries, whose index arithmetic is then shared by more threads).
+// k_finalize / here: 4x4 cluster, 64 frequencies, 4 momenta, 13 transfers 0.39 /
+// 0.36 ms, 32: 1.29 / 0.76, 64: 4.6 / 1.5, but 11: 0.32 / 0.38; 3x3, 16
+// frequencies, 9 momenta, 9 transfers 0.020 / 0.014, but 17 frequencies, 7
+// momenta, 5 transfers 0.025 / 0.029.
+bool finalize_wide(const G4Dims& d) { return d.Nwex > 12 || (d.Nwex > 8 && d.Nc < 12); }
+
+template <bool PAIR>
+__global__ void __launch_bounds__(256) k_finalize_wide(const double2* __restrict__ acc, double inv_s,
+                                                       double2* __restrict__ out, G4Dims d, int KC, int n2_0,
+                                                       int q0, long long out_plane) {
+    extern __shared__ double2 tileF[];  // [KC][Nc][Nwex + 1]
+    const int n1 = blockIdx.x, n2l = blockIdx.y, q = q0 + blockIdx.z;
+    const int n2 = n2_0 + n2l;
+    const int Nc = d.Nc, Nw2 = d.Nw2, Nwex = d.Nwex, ld = Nwex + 1;
+    for (int k20 = 0; k20 < Nc; k20 += KC) {
+        const int kc = min(KC, Nc - k20);
+        const int cnt = kc * Nc * Nwex;
+        for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+            const int r = t / Nwex, m = t - r * Nwex;
+            const int k2l = r / Nc, k1 = r - k2l * Nc;
+            const size_t K1 = (size_t)k1 * Nw2 + n1, K2 = (size_t)(k20 + k2l) * Nw2 + n2;
+            tileF[r * ld + m] = acc_value<PAIR>(acc, (K1 * d.N + K2) * d.NQ + (size_t)q * Nwex + m);
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+            const int m = t / (kc * Nc), r = t - m * (kc * Nc);   // r = (k2l, k1), k1 fastest
+            const double2 v = tileF[r * ld + m];
+            out[(size_t)m * out_plane + (((size_t)n2l * Nw2 + n1) * d.Nkex + q) * Nc * Nc +
+                (size_t)k20 * Nc + r] = make_double2(v.x * inv_s, v.y * inv_s);
         }
         __syncthreads();
     }
@@ -579,18 +622,35 @@ cudaError_t launch_update_fp64(const double2* G, const G4Signs& signs, int stage
 cudaError_t launch_finalize(const double2* acc, bool pair, double inv_s, double2* out,
                             const G4Dims& d, int n2_0, int n2_cnt, long long out_plane, int q0,
                             int nq, const float2* scr, const double2* scr0, cudaStream_t s) {
+    const int NR = d.Nc * d.Nc;
+    const size_t plane = (size_t)d.Nc * (d.Nwex + 1) * sizeof(double2);   // one k2
+    if (!scr && finalize_wide(d) && plane <= kFinWideMax) {
+        const int KC = (int)std::min<size_t>(d.Nc, std::max<size_t>(1, kFinWideBytes / plane));
+        auto* k = pair ? k_finalize_wide<true> : k_finalize_wide<false>;
+        if (KC * plane > 48 * 1024) {
+            cudaError_t e = raise_smem_limit(k);
+            if (e != cudaSuccess) return e;
+        }
+        k<<<dim3(d.Nw2, n2_cnt, nq), 256, KC * plane, s>>>(acc, inv_s, out, d, KC, n2_0, q0, out_plane);
+        return cudaGetLastError();
+    }
     // transfers per block: a 128-byte run, or one momentum's (NJ * kFinN2 is at
     // most kFinThreads: Nwex <= 64)
     const int TQ = std::min(nq, std::max(1, kFinNJ / d.Nwex));
     const int NJ = TQ * d.Nwex, ld = NJ | 1;
     const size_t per = (size_t)kFinN2 * ld * sizeof(double2);
-    int RC = (int)std::min<size_t>((size_t)d.Nc * d.Nc, std::max<size_t>(1, kFinBytes / per));
-    if (RC >= 8) RC = RC / 8 * 8;
+    const long long blocks = (long long)d.Nw2 * ((n2_cnt + kFinN2 - 1) / kFinN2) * ((nq + TQ - 1) / TQ);
+    // pairs per chunk: all of them, or equal chunks of whole 128-byte lines
+    int RC = (int)std::min<size_t>(NR, std::max<size_t>(1, kFinBytes / per));
+    if (RC < NR && RC >= 8) {
+        RC = RC / 8 * 8;
+        const int n = (NR + RC - 1) / RC;
+        RC = ((NR + n - 1) / n + 7) / 8 * 8;
+    }
     // the chunks are dealt to enough blocks to fill the GPU several times over
     // (8x8 cluster, 32 frequencies: 15.0 ms with a group's blocks undivided, 11.0
     // divided)
-    const long long blocks = (long long)d.Nw2 * ((n2_cnt + kFinN2 - 1) / kFinN2) * ((nq + TQ - 1) / TQ);
-    const long long chunks = ((long long)d.Nc * d.Nc + RC - 1) / RC;
+    const long long chunks = ((long long)NR + RC - 1) / RC;
     const int nsplit = (int)std::min<long long>(std::min<long long>(chunks, 256), (kFinBlocks + blocks - 1) / blocks);
     const dim3 grid(d.Nw2, (n2_cnt + kFinN2 - 1) / kFinN2, (nq + TQ - 1) / TQ * nsplit);
     auto* k = pair ? k_finalize<true, false> : scr ? k_finalize<false, true> : k_finalize<false, false>;

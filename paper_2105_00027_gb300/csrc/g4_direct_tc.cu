@@ -546,7 +546,8 @@ struct DirectPlan {
     int fill = 0;        // measurements in the window
     int batches = 0;     // full batches the window holds
     int Kst = 0;         // row stride of the split planes (2 * Bw elements)
-    int nQg = 0;         // transfers per group (whole momenta where Nwex allows it)
+    int nQg = 0;         // transfers per group
+    bool whole = false;  // groups of whole momenta: g4_finalize takes the window along
     bool f16 = true;     // FP16 (else TF32) hi/lo planes
     float2* araw = nullptr;   // [NQ][N][Bw]
     float2* braw = nullptr;
@@ -620,7 +621,14 @@ g4_status direct_prepare(g4_ctx* h) {
     X->f16 = h->opt.operands == G4_OPERANDS_FP16;
     X->Bw = (F * h->batch + 31) / 32 * 32;   // 2 Bw: a whole number of 64-element stages
     X->Kst = 2 * X->Bw;
-    X->nQg = std::min(d.Nwex <= kGroupQ ? kGroupQ / d.Nwex * d.Nwex : kGroupQ, d.NQ);
+    // whole momenta where the export takes the last window: not for more than 8
+    // transfers on clusters of less than twelve sites, where groups of less than
+    // sixteen transfers cost more than the accumulator's read-modify-write (3x3, 34
+    // frequencies, 11 transfers, 9 momenta: GEMM, merge and export 0.26 ms, 0.31
+    // with the window in the export; 5x3, 50 frequencies: 1.25 and 1.13)
+    const bool whole = d.Nwex <= kGroupQ && (d.Nwex <= 8 || d.Nc >= 12);
+    X->nQg = std::min(whole ? kGroupQ / d.Nwex * d.Nwex : kGroupQ, d.NQ);
+    X->whole = whole;
     g4_status st;
     const size_t raw = (size_t)d.NQ * d.N * X->Bw;
     if ((st = dalloc(h, &X->araw, raw)) != G4_OK) return st;
@@ -759,7 +767,7 @@ g4_status direct_flush(g4_ctx* h) {
 
 bool direct_finalize_ok(const g4_ctx* h) {
     const DirectPlan* X = (const DirectPlan*)h->dplan;
-    return X && X->fill > 0 && X->nQg % h->d.Nwex == 0 && h->opt.accum != G4_ACCUM_F32PAIR;
+    return X && X->fill > 0 && X->whole && h->opt.accum != G4_ACCUM_F32PAIR;
 }
 
 g4_status direct_finalize(g4_ctx* h, double inv_s, double2* out) {
