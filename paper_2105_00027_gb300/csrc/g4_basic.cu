@@ -69,9 +69,13 @@ __global__ void __launch_bounds__(256) k_build_G_fp64(const void* __restrict__ M
 // CH (see g4.h).  Block row K1 = blockIdx.y; groups of RS lanes run over (K2, Q)
 // with Q fastest, so the accumulator read-modify-write, once per batch, is
 // coalesced; the lanes of a group share out the measurements and add up their
-// sums by shuffles.  The kernel of shapes the tiled one does not take (RS = 1)
-// and of small problems, where a lane's chain over the measurements is the
-// whole time (1024 entries, 16 measurements: 29 us with RS = 1, 5 with 16).
+// sums by shuffles.  The kernel of shapes the tiled one does not take (RS = 1,
+// measurement by measurement onto the accumulator: sums apart from it are two
+// more operations on the FP64 pipe, which bounds the kernel; one measurement at a
+// time on the 4x4 cluster with 32 frequencies, particle-particle, 0.25 ms with
+// them, 0.22 without) and of small problems, where a lane's chain over the
+// measurements is the whole time (1024 entries, 16 measurements: 29 us with RS =
+// 1, 5 with 16).
 template <int CH, int RS>
 __global__ void k_update_fp64(const double2* __restrict__ Gb, const __grid_constant__ G4Signs signs,
                               int staged, double2* __restrict__ acc, const int* __restrict__ kadd,
@@ -92,6 +96,7 @@ __global__ void k_update_fp64(const double2* __restrict__ Gb, const __grid_const
         const int q = Qi / d.Nwex, m = d.m0 + Qi - q * d.Nwex;   // m: the transfer frequency
         const int k2 = K2 / d.Nw2, n2 = K2 - k2 * d.Nw2;
         double2 o = make_double2(0.0, 0.0);
+        if (RS == 1 && idx0 < per) o = row[idx];
         for (int r = sub; r < staged; r += RS) {
             const double2* G = Gb + (size_t)(2 * r) * NN;
             const double sign = signs.s[r];
@@ -111,7 +116,8 @@ __global__ void k_update_fp64(const double2* __restrict__ Gb, const __grid_const
                     }
                 }
             } else {
-                const bool v1 = n1 + m < d.Nw2, v2 = n2 + m < d.Nw2;
+                // an entry off the grid stays zero
+                if (n1 + m >= d.Nw2 || n2 + m >= d.Nw2) break;
                 const int K1Q = kadd[k1 * d.Nc + q] * d.Nw2 + n1 + m;
                 const int K2Q = kadd[k2 * d.Nc + q] * d.Nw2 + n2 + m;
                 double2 a = make_double2(0, 0), b = make_double2(0, 0), ex = make_double2(0, 0);
@@ -120,24 +126,18 @@ __global__ void k_update_fp64(const double2* __restrict__ Gb, const __grid_const
                     const double2* g = G + sp * NN;
                     const double wgt = (CH == G4_PH_MAGNETIC && sp) ? -1.0 : 1.0;
                     if (CH != G4_PH_TRANSVERSE) {
-                        if (v1) {
-                            const double2 t = g[(size_t)K1Q * d.N + K1];
-                            a.x += wgt * t.x;
-                            a.y += wgt * t.y;
-                        }
-                        if (v2) {
-                            const double2 t = g[(size_t)K2 * d.N + K2Q];
-                            b.x += wgt * t.x;
-                            b.y += wgt * t.y;
-                        }
+                        double2 t = g[(size_t)K1Q * d.N + K1];
+                        a.x += wgt * t.x;
+                        a.y += wgt * t.y;
+                        t = g[(size_t)K2 * d.N + K2Q];
+                        b.x += wgt * t.x;
+                        b.y += wgt * t.y;
                     }
-                    if (v1 && v2) {
-                        // transverse pairs the opposite spin in the G(K2,K1) factor
-                        const double2* gx = CH == G4_PH_TRANSVERSE ? G + (1 - sp) * NN : g;
-                        const double2 t = cmul(gx[(size_t)K2 * d.N + K1], g[(size_t)K1Q * d.N + K2Q]);
-                        ex.x += t.x;
-                        ex.y += t.y;
-                    }
+                    // transverse pairs the opposite spin in the G(K2,K1) factor
+                    const double2* gx = CH == G4_PH_TRANSVERSE ? G + (1 - sp) * NN : g;
+                    const double2 t = cmul(gx[(size_t)K2 * d.N + K1], g[(size_t)K1Q * d.N + K2Q]);
+                    ex.x += t.x;
+                    ex.y += t.y;
                 }
                 const double2 ab = cmul(a, b);
                 term = make_double2(ab.x - ex.x, ab.y - ex.y);
@@ -150,7 +150,7 @@ __global__ void k_update_fp64(const double2* __restrict__ Gb, const __grid_const
             o.x += __shfl_xor_sync(0xffffffffu, o.x, w);
             o.y += __shfl_xor_sync(0xffffffffu, o.y, w);
         }
-        if (sub == 0 && idx0 < per) row[idx] = make_double2(row[idx].x + o.x, row[idx].y + o.y);
+        if (sub == 0 && idx0 < per) row[idx] = RS == 1 ? o : make_double2(row[idx].x + o.x, row[idx].y + o.y);
     }
 }
 
@@ -206,7 +206,9 @@ __global__ void __launch_bounds__(kTileF * kTileF) k_update_fp64_tiled(
             const double2* G = Gb + (size_t)(2 * r) * NN;
             const double sign = signs.s[r];
             __syncthreads();  // the previous tiles are no longer read
-            // G(K2, K1) of the tile (the transverse channel pairs the opposite spin)
+            // G(K2, K1) of the tile (the transverse channel pairs the opposite spin);
+            // a single measurement's stays over the transfers
+            if (staged > 1 || q == 0)
             for (int t = threadIdx.x; t < 2 * kTileF * kTileF; t += blockDim.x) {
                 const int sp = t / (kTileF * kTileF), u = t % (kTileF * kTileF);
                 const int a2 = u / kTileF, a1 = u % kTileF;
@@ -550,7 +552,23 @@ __global__ void k_clear_unset(double2* __restrict__ acc, long long E, const unsi
         acc[i] = make_double2(0.0, 0.0);
 }
 
+// Whether the tiled update takes the shape: from 2^18 entries on (below, a launch
+// of it is a chain of barriers over transfers and measurements in a few blocks),
+// when enough of its frequency tiles lies on the grid (Nw2^2 of the tiles' area;
+// the opposite-spin channel, without the direct term, has less to share in a
+// tile).  16 measurements, simple / tiled, ms: 3x3 cluster, 9 momenta, magnetic, 4
+// transfers: 20 frequencies (0.39 of the tiles) 0.99 / 1.64, 24 (0.56) 1.41 /
+// 1.64, 28 (0.77) 1.91 / 1.65; 2x2, 8 transfers, 50 (0.61) 1.06 / 0.92;
+// transverse: 28 1.09 / 1.14, 3 transfers, 40 (0.69) 1.65 / 1.51, 2 transfers,
+// 48 (1) 1.59 / 1.14; one measurement at a time 28 1.19 / 1.45, 40 1.76 / 1.76.
 constexpr long long kTiledMinEntries = 1 << 18;
+bool tiled_wanted(const G4Dims& d) {
+    if (d.ch == G4_PP_UPDOWN || d.Nwex > kTileWex || (long long)d.Nc * d.Nc > 65535 || d.E < kTiledMinEntries)
+        return false;
+    const int side = (d.Nw2 + kTileF - 1) / kTileF * kTileF;
+    const double fill = (double)d.Nw2 * d.Nw2 / ((double)side * side);
+    return d.ch == G4_PH_TRANSVERSE ? d.Nwex > 1 && fill >= 0.78 : fill >= 0.6;
+}
 
 }  // namespace
 
@@ -570,10 +588,7 @@ template <int CH>
 cudaError_t update_fp64(const double2* G, const G4Signs& signs, int staged, double2* acc,
                         const int* kadd, const int* ksub, const G4Dims& d, const unsigned* only_if,
                         cudaStream_t s) {
-    // the tiled kernel from 2^18 entries on; below, a launch of it is a chain of
-    // barriers over transfers and measurements in a few blocks
-    if (CH != G4_PP_UPDOWN && d.Nwex <= kTileWex && (long long)d.Nc * d.Nc <= 65535 &&
-        d.E >= kTiledMinEntries) {
+    if (tiled_wanted(d)) {
         const int nt = (d.Nw2 + kTileF - 1) / kTileF;
         const int WX = kTileF + d.Nwex - 1;
         const size_t smem = (2 * (size_t)WX * (WX + 1) + 2 * kTileF * (kTileF + 1) +
