@@ -619,6 +619,15 @@ cudaError_t update_fp64(const double2* G, const G4Signs& signs, int staged, doub
 }
 }  // namespace
 
+double update_fp64_ps(const G4Dims& d) {
+    if (d.ch == G4_PP_UPDOWN) return 25.5;
+    const bool trans = d.ch == G4_PH_TRANSVERSE;
+    if (!tiled_wanted(d)) return trans ? 30.0 : 52.0;
+    const int side = (d.Nw2 + kTileF - 1) / kTileF * kTileF;
+    const double fill = (double)d.Nw2 * d.Nw2 / ((double)side * side);
+    return (trans ? 15.5 + 6.0 / d.Nwex : 22.5 + 10.0 / d.Nwex) / fill;
+}
+
 cudaError_t launch_update_fp64(const double2* G, const G4Signs& signs, int staged, double2* acc,
                                const int* kadd, const int* ksub, const G4Dims& d,
                                const unsigned* only_if, cudaStream_t s) {

@@ -795,6 +795,7 @@ __global__ void __launch_bounds__(256) k_merge64(const double2* __restrict__ scr
 
 // ------------------------------------------------------------------ host
 struct F64Plan {
+    double tiles = 0;          // exchange tiles of a batch
     int kb = 0, nb = 0, W = 0, pb = 0, nkb = 0, npb = 0, N = 0;
     int Jh = 0, J = 0, Bp = 0, gcap = 0, nQg = 0;
     std::vector<int> gd0, gdn, gw0, gwn;   // per group: diagonals, work entries
@@ -853,9 +854,12 @@ bool encode_maps(const G4Dims& d, F64Plan& X) {
     return make(&X.dA, 4, X.ab, dd, ds, da) && make(&X.dB, 4, bside, dd, ds, db);
 }
 
-// The tile shape (kb x nb rows, pb x W columns) with the least time by a model
-// in clocks, over all diagonals: the larger of the MMAs (shared-memory reads of
-// A and B at 128 B per clock; nsteps of 16 values of K) and the epilogue.
+// Clocks of one exchange tile of N columns and nsteps x 16 values of K: measured
+// over shapes of one to 256 sites and 2 to 128 frequencies, within a tenth.
+double tile_clocks(int N, int nsteps) { return 8000.0 + 10.5 * nsteps * (kARows + N); }
+
+// The tile shape (kb x nb rows, pb x W columns) with the least time over all
+// diagonals.
 bool choose_tile(const G4Dims& d, int nsteps, F64Plan& X) {
     double best = 1e300;
     for (int nb = 1; nb <= 16 && nb <= d.Nw2; ++nb) {
@@ -868,7 +872,7 @@ bool choose_tile(const G4Dims& d, int nsteps, F64Plan& X) {
                 const int N = (W * pb + 15) / 16 * 16;
                 if (N > kMaxN || f_smem(N, pb * d.Nwex) > kMaxSmem) break;
                 const int nkb = (d.Nc + kb - 1) / kb, npb = (d.Nc + pb - 1) / pb;
-                const double cost = blocks * nkb * npb * (std::max((kARows + N) / 4.0 * 36 * nsteps, 1700.0 + 130.0 * N) + 500.0);
+                const double cost = blocks * nkb * npb * tile_clocks(N, nsteps);
                 if (cost < best) {
                     best = cost;
                     X.kb = kb;
@@ -878,6 +882,7 @@ bool choose_tile(const G4Dims& d, int nsteps, F64Plan& X) {
                     X.nkb = nkb;
                     X.npb = npb;
                     X.N = N;
+                    X.tiles = blocks * nkb * npb * d.Nc;
                 }
             }
     }
@@ -901,14 +906,33 @@ size_t plan_bytes(const G4Dims& d, int batch) {
     return std::min<size_t>(std::max<size_t>(held, (size_t)512 << 20), (size_t)4 << 30);
 }
 
+// Whether a batch of `staged` measurements takes less time here than in the plain
+// kernels, by times measured on the shapes of tile_clocks and 4 to 64
+// measurements: the work here does not shrink with the transfer momenta (every
+// tile holds all of them) nor, below 16 measurements, with the batch.  In
+// microseconds; where the two sides are not near each other the estimates are
+// within a quarter.  (By the number of element-updates alone, from 4e6 on, 16x16
+// sites with 2 frequencies and 4 momenta took 2.7 ms for 16 measurements, 0.9 in
+// the plain kernel.)
+bool faster_here(const G4Dims& d, const F64Plan& X, int staged, int sms, size_t ngroups) {
+    const double N2 = (double)d.N * d.N;
+    const int live = X.Jh > 16 ? (staged + 31) / 32 * 32 : 16;
+    const double exchange = 30.0 + X.tiles / sms * tile_clocks(X.N, live / 4) / 1900.0;
+    // the check and the pack: G read twice, digits written; TB/s
+    const double rate = 3.6 * d.Nw2 / (d.Nw2 + 3.0) / (ngroups == 1 ? 1.0 : d.Nw2 < 24 ? 1.6 : 1.2);
+    const double pack = 20.0 + N2 * (64.0 * staged + 96.0 * live) / rate * 1e-6;
+    double direct = 0.0;
+    if (has_direct(d.ch))
+        direct = 25.0 * ((d.NQ + X.nQg - 1) / X.nQg) + d.NQ * N2 * (12.0 + 0.4 * staged) * 1e-6;
+    return exchange + pack + direct < 5.0 + (double)d.E * staged * update_fp64_ps(d) * 1e-6;
+}
+
 }  // namespace
 
 void f64tc_prepare(g4_ctx* h) {
     const G4Dims& d = h->d;
-    // below kF64tcMinUpdates element-updates a batch is some 0.1 ms of the plain
-    // kernel; a memory limit or a wait budget of the caller's is kept as it was
-    if (h->opt.mem_limit > 0 || h->opt.timeout_cycles > 0) return;
-    if (d.Nwex > kMaxWex || (double)d.E * h->batch < kF64tcMinUpdates) return;
+    // a memory limit or a wait budget of the caller's is kept as it was
+    if (h->opt.mem_limit > 0 || h->opt.timeout_cycles > 0 || d.Nwex > kMaxWex) return;
     F64Plan* X = new (std::nothrow) F64Plan();
     if (!X) return;
     const bool cross = d.ch == G4_PH_TRANSVERSE || d.ch == G4_PP_UPDOWN;
@@ -937,7 +961,9 @@ void f64tc_prepare(g4_ctx* h) {
         const size_t fit = std::min<size_t>((budget - direct_b) / per_diag, 65535);
         const size_t ng = (dl.size() + fit - 1) / fit;
         X->gcap = (int)std::min<size_t>(fit, ((dl.size() + ng - 1) / ng + 1) / 2 * 2);
-        ok = ok && (size_t)X->gcap * kDig < ((size_t)1 << 31);
+        ok = ok && (size_t)X->gcap * kDig < ((size_t)1 << 31) &&
+             cudaDeviceGetAttribute(&X->sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess &&
+             faster_here(d, *X, h->batch, X->sms, ng);
     }
     std::vector<int4> work;
     std::vector<int> pos0(d.Nc, -1);
@@ -987,8 +1013,7 @@ void f64tc_prepare(g4_ctx* h) {
          cudaMemcpy(X->work, work.data(), work.size() * sizeof(int4), cudaMemcpyHostToDevice) == cudaSuccess &&
          cudaMemcpy(X->pos0, pos0.data(), pos0.size() * sizeof(int), cudaMemcpyHostToDevice) == cudaSuccess &&
          encode_maps(d, *X) && raise_smem_limit(k_spread) == cudaSuccess && raise_smem_limit(k_gemm_digits<0>) == cudaSuccess &&
-         raise_smem_limit(k_gemm_digits<1>) == cudaSuccess && raise_smem_limit(k_gemm_digits<2>) == cudaSuccess &&
-         cudaDeviceGetAttribute(&X->sms, cudaDevAttrMultiProcessorCount, h->device) == cudaSuccess;
+         raise_smem_limit(k_gemm_digits<1>) == cudaSuccess && raise_smem_limit(k_gemm_digits<2>) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         f_free(X);
@@ -1007,7 +1032,9 @@ void f64tc_release(g4_ctx* h) {
 
 bool f64tc_wanted(const g4_ctx* h, int staged) {
     // fewer than four measurements: k_spread has no quarter to spare
-    if (!h->f64tc || h->f64_plain || staged < 4 || (double)h->d.E * staged < kF64tcMinUpdates) return false;
+    if (!h->f64tc || h->f64_plain || staged < 4) return false;
+    const F64Plan* X = (const F64Plan*)h->f64tc;
+    if (staged < h->batch && !faster_here(h->d, *X, staged, X->sms, X->gd0.size())) return false;
     // the sign factors must stay in the digits' exponent range
     for (int r = 0; r < staged; ++r) {
         const double a = std::fabs(h->slot_sign[r]);

@@ -202,9 +202,11 @@ cudaError_t launch_update_fp64(const double2* G, const G4Signs& signs, int stage
                                const int* kadd, const int* ksub, const G4Dims& d,
                                const unsigned* only_if, cudaStream_t s);
 
+// its time per element-update in picoseconds, measured on problems that fill the GPU
+double update_fp64_ps(const G4Dims& d);
+
 // FP64 path, a batch's update on tensor cores (g4_fp64_tc.cu): prepare leaves
 // h->f64tc null where the path does not apply (or its memory is not there)
-constexpr double kF64tcMinUpdates = 4e6;
 void f64tc_prepare(g4_ctx* h);
 bool f64tc_wanted(const g4_ctx* h, int staged);
 g4_status f64tc_run(g4_ctx* h, int staged);

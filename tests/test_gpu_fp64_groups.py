@@ -43,8 +43,10 @@ def test_slab(channel):
     whole, _, h = run_lib(p, M, G0, s, "fp64", channel=channel)
     h.close()
     for first, count in ((0, 3), (2, 3)):
-        assert p.entries // p.Nwex * count * p.R >= 4e6     # the tensor-core form's threshold
-        part, _, h = run_lib(p, M, G0, s, "fp64", channel=channel, wex_slab=(first, count))
+        h = ensure_built().G4.for_problem(p, precision="fp64", channel=channel, wex_slab=(first, count))
+        h.profile()
+        part, _, h = run_lib(p, M, G0, s, "fp64", channel=channel, handle=h)
+        assert h.profile_read("exchange")[1] > 0     # the tensor-core form
         h.close()
         assert np.array_equal(part.reshape(count, -1), whole.reshape(p.Nwex, -1)[first:first + count])
 

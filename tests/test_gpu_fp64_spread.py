@@ -63,9 +63,11 @@ def check(M, G0, s, channel):
     G = torch.stack([g4.build_G(Md[r].contiguous(), G0d) for r in range(R)])
     ref, S = reference(P, G, s, channel)
     h = g4.G4.for_problem(P, precision="fp64", channel=channel)
+    h.profile()
     for r in range(R):
         h.compute_G(Md[r], G0d, float(s[r]))
     got, _ = h.finalize()
+    assert h.profile_read("exchange")[1] > 0     # the tensor-core form (unless its check leaves the batch)
     h.close()
     err = (got.reshape(ref.shape) - ref).abs()
     assert bool((err <= 4 * (2 * R + 8) * 2.0 ** -53 * S).all()), float((err / S.clamp_min(1e-300)).max())
