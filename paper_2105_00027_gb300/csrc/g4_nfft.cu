@@ -790,6 +790,14 @@ struct GroupCfg {
             g = dim3((unsigned)((d.Nw2 + RT - 1) / RT), (unsigned)((nmax + CT - 1) / CT), 2);
         else
             g = dim3((unsigned)((d.N + RT - 1) / RT), (unsigned)((d.Nw2 + CT - 1) / CT), 2);
+        // FP64 launches are plain: started programmatically, grids of less than a
+        // wave were spread worse over the SMs (6x6 sites, 8 frequencies, 300
+        // vertices: a transform 62 us, 83 programmatically; 8x8, 4 frequencies 74 and
+        // 90), where the FP32 ones gain 2 to 10 us in every shape
+        if constexpr (std::is_same<C, double2>::value) {
+            k_nfft_group<C, LEFT, RT, CT, RB, CB><<<g, nw * 32, smem(d.Nc, nw), st>>>(a, tw, E, Mr, Tm, out, scale);
+            return cudaGetLastError();
+        }
         return launch_pdl(k_nfft_group<C, LEFT, RT, CT, RB, CB>, g, dim3(nw * 32), smem(d.Nc, nw), st, a, tw,
                           E, Mr, Tm, out, scale);
     }
