@@ -21,11 +21,13 @@ __device__ __forceinline__ double2 cmul(double2 a, double2 b) {
 
 // G[sp][i][j] = G0[sp][i] d_ij - G0[sp][i] M[sp][i][j] G0[sp][j], FP64.  A
 // block takes kBuildU blocks of columns of one row (no division per entry,
-// kBuildU independent loads in flight); flag (may be null): see
-// launch_build_G_fp64, tested on the exponent fields.
-constexpr int kBuildU = 4;
+// kBuildU independent loads in flight); FLAG: see launch_build_G_fp64, tested on
+// the exponent fields.  Bound by the FP64 pipe and, with the test, the issue
+// slots: 20 builds of N = 1000 took 0.95 ms with one entry per thread, 1.00 with
+// the test always made and four, 0.83 with two and the test where it is used.
+constexpr int kBuildU = 2;
 
-template <bool M64>
+template <bool M64, bool FLAG>
 __global__ void __launch_bounds__(256) k_build_G_fp64(const void* __restrict__ M,
                                                       const double2* __restrict__ G0,
                                                       double2* __restrict__ G, int N,
@@ -54,7 +56,8 @@ __global__ void __launch_bounds__(256) k_build_G_fp64(const void* __restrict__ M
             double2 v = cmul(cmul(ngi, make_double2(m[u].x, m[u].y)), gj[u]);
             if (i == j) v = make_double2(v.x + gi.x, v.y + gi.y);
             G[(size_t)row * N + j] = v;
-            // on the exponent fields, off the FP64 pipe (which bounds this kernel)
+            if constexpr (!FLAG) continue;
+            // off the FP64 pipe
             const long long bx = __double_as_longlong(v.x) & 0x7FFFFFFFFFFFFFFFll;
             const long long by = __double_as_longlong(v.y) & 0x7FFFFFFFFFFFFFFFll;
             constexpr unsigned lo = (unsigned)(1023 - kF64tcExp) << 20, span = (unsigned)(2 * kF64tcExp) << 20;
@@ -62,7 +65,7 @@ __global__ void __launch_bounds__(256) k_build_G_fp64(const void* __restrict__ M
                   ((unsigned)(by >> 32) - lo > span && by != 0);
         }
     }
-    if (flag && bad) *flag = 1u;
+    if (FLAG && bad) *flag = 1u;
 }
 
 // The staged measurements' FP64 update of every accumulator entry, for channel
@@ -576,10 +579,9 @@ cudaError_t launch_build_G_fp64(const void* M, bool m64, const double2* G0, doub
                                 unsigned* flag, cudaStream_t s) {
     const int bx = N >= 256 ? 256 : (N + 31) / 32 * 32;
     const dim3 grid((N + kBuildU * bx - 1) / (kBuildU * bx), std::min(2LL * N, 65535LL));
-    if (m64)
-        k_build_G_fp64<true><<<grid, bx, 0, s>>>(M, G0, G, N, flag);
-    else
-        k_build_G_fp64<false><<<grid, bx, 0, s>>>(M, G0, G, N, flag);
+    auto* k = m64 ? (flag ? k_build_G_fp64<true, true> : k_build_G_fp64<true, false>)
+                  : (flag ? k_build_G_fp64<false, true> : k_build_G_fp64<false, false>);
+    k<<<grid, bx, 0, s>>>(M, G0, G, N, flag);
     return cudaGetLastError();
 }
 
