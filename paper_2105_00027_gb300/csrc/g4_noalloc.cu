@@ -91,7 +91,8 @@ __device__ __forceinline__ void na_cfma(double2& t, double2 a, double2 b) {
     t.y = fma(a.y, b.x, t.y);
 }
 
-__global__ void __launch_bounds__(kNaThreads) k_na_update(const double2* __restrict__ G, double sign,
+template <bool DEAL>
+__global__ void __launch_bounds__(kNaThreads, 3) k_na_update(const double2* __restrict__ G, double sign,
                                                           double2* __restrict__ acc, int Nc, int Lx,
                                                           int Nw2, int Nwex, int Nkex, int gp, int nm) {
     __shared__ double2 sa[kNaM * kNaThreads], sb[kNaM * kNaThreads];   // [m][group][k]
@@ -105,8 +106,10 @@ __global__ void __launch_bounds__(kNaThreads) k_na_update(const double2* __restr
         y -= y >= Ly ? Ly : 0;
         return x + Lx * y;
     };
-    const int zm = blockIdx.z % nm, zp = blockIdx.z / nm, np = gridDim.z / nm;
-    for (int m0 = zm * kNaM; m0 < Nwex; m0 += nm * kNaM) {
+    const int zm = DEAL ? blockIdx.z % nm : 0, mstep = DEAL ? nm * kNaM : kNaM;
+    const int t0 = DEAL ? blockIdx.z / nm * blockDim.x + threadIdx.x : threadIdx.x;
+    const int tstep = DEAL ? gridDim.z / nm * blockDim.x : blockDim.x;
+    for (int m0 = zm * kNaM; m0 < Nwex; m0 += mstep) {
         __syncthreads();
         for (int t = threadIdx.x; t < ng * Nc; t += blockDim.x) {
             const int g = t / Nc, k = t - g * Nc;
@@ -131,7 +134,7 @@ __global__ void __launch_bounds__(kNaThreads) k_na_update(const double2* __restr
             }
         }
         __syncthreads();
-        for (int t = zp * blockDim.x + threadIdx.x; t < ng * N2; t += np * blockDim.x) {
+        for (int t = DEAL ? t0 : threadIdx.x; t < ng * N2; t += DEAL ? tstep : blockDim.x) {
             const int g = t / N2, r = t - g * N2, k2 = r / Nc, k1 = r - k2 * Nc;
             const int n1 = (g0 + g) / Nkex, q = (g0 + g) - n1 * Nkex;
             const int lim = min(Nwex, Nw2 - max(n1, n2)) - m0;   // transfers on the grid
@@ -254,8 +257,8 @@ extern "C" g4_status g4_update_noalloc(int Nc, int lx, int Nw, int Nwex, int Nke
     const int nm = std::min((Nwex + kNaM - 1) / kNaM, (kNaBlocks + blocks2 - 1) / blocks2);
     const int np = std::min((std::min(gp, groups) * Nc * Nc + kNaThreads - 1) / kNaThreads,
                             (kNaBlocks + blocks2 * nm - 1) / (blocks2 * nm));
-    k_na_update<<<dim3(bx, 2 * Nw, nm * np), kNaThreads, 0, s>>>(G, sign, (double2*)acc, Nc, Lx, 2 * Nw, Nwex, Nkex,
-                                                                 gp, nm);
+    auto* k = nm * np > 1 ? k_na_update<true> : k_na_update<false>;
+    k<<<dim3(bx, 2 * Nw, nm * np), kNaThreads, 0, s>>>(G, sign, (double2*)acc, Nc, Lx, 2 * Nw, Nwex, Nkex, gp, nm);
     e = cudaGetLastError();
     if (e != cudaSuccess) return na_fail(G4_ERR_CUDA, std::string("update launch: ") + cudaGetErrorString(e));
     return G4_OK;
