@@ -12,7 +12,7 @@ Printed JSON line: the metric of the G4 workload (element-updates/s = E*R/t),
 the roofline of the dominant kernel (the exchange-type term: on tensor cores
 bound by the HBM stream of its FP64 accumulator and operands, on CUDA cores by
 the FP32 ALUs), the plain
-FP64 per-measurement GPU path on the same problem dimensions for comparison,
+FP64 GPU path on the same problem dimensions for comparison,
 an end-to-end number with host inputs, the same run fed from vertex
 configurations (the transform to M before the path, with its own FP32 ALU
 roofline), the oracle on the host cores, and the SM clocks sampled during the

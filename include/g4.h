@@ -321,11 +321,14 @@ typedef enum {
     G4_K_PACK = 1,         /* direct-term operands of a batch into the window */
     G4_K_DIRECT = 2,       /* direct-term GEMM of a transfer group (tensor cores) */
     G4_K_EXCHANGE = 3,     /* exchange-type term + FP64 accumulate (either kernel) */
-    G4_K_UPDATE_FP64 = 4,  /* plain FP64 per-measurement update */
+    G4_K_UPDATE_FP64 = 4,  /* plain FP64 update of a batch (after the tensor-core form: only
+                              if the batch was left to it) */
     G4_K_FINALIZE = 5,     /* normalisation + export transpose */
-    G4_K_PACK_EXCHANGE = 6,/* exchange operand pack (tensor-core exchange) */
+    G4_K_PACK_EXCHANGE = 6,/* exchange operand pack (tensor-core exchange; FP64: digits and
+                              the check before them) */
     G4_K_NFFT = 7,         /* vertex configuration -> M (sort, phases, both products) */
-    G4_K_DIRECT_SPLIT = 8, /* direct-term TF32 hi/lo planes of a transfer group */
+    G4_K_DIRECT_SPLIT = 8, /* direct-term operand planes of a transfer group (FP16 or TF32
+                              pairs; FP64: digits) */
     G4_K_DIRECT_MERGE = 9, /* direct-term scratch added to the FP64 accumulator */
     G4_K_COUNT = 10
 } g4_kernel_kind;

@@ -1,5 +1,5 @@
 // C ABI of the G4 library: handle lifecycle, argument checking, batching and
-// dispatch to the FP64 plain path or the mixed-precision path.
+// dispatch to the FP64 or the mixed-precision path.
 #include <algorithm>
 #include <atomic>
 #include <cstdint>

@@ -2,8 +2,8 @@
 //   * G build, G = G0 d - G0 M G0 (Sec. 2), in the natural layout (FP64 path,
 //     standalone g4_build_G) and in the diagonal-major complex64 layout the
 //     mixed path consumes;
-//   * the plain FP64 per-measurement update of the particle-hole magnetic G4
-//     (the accumulation of Eq. (1), Sec. 2.1);
+//   * the plain FP64 update of G4 with a batch of measurements (the
+//     accumulation of Eq. (1), Sec. 2.1);
 //   * the final normalisation by the sign sum and the transpose to the
 //     exported layout.
 #include <algorithm>

@@ -1042,7 +1042,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         // acc[K1][K2][q][0..Nwex) into the warp's run buffer in shared memory, and
         // the pair's first lane adds the run to the accumulator with one
         // asynchronous bulk reduction (performed at L2, so no load round trip
-        // holds up the epilogue).  Two run buffers per warp alternate; before a
+        // holds up the epilogue).  kRunBufs run buffers per warp take turns; before a
         // buffer is rewritten its reductions must have read it.  The partial
         // sums of a split tile (D = 0) go to the same entries, so there every
         // reduction completes before the next one is issued (a fixed order of
@@ -1173,7 +1173,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                                                      (uint32_t)(16 * mlim));
                             }
                         }
-                        bulk_commit();  // one group per pass, so that "all but the last" is the other buffer
+                        bulk_commit();  // one group per pass, for the wait above
                     }
                     wb = wb + 1 == kRunBufs ? 0 : wb + 1;
                 }
