@@ -166,9 +166,13 @@ __global__ void k_update_fp64(const double2* __restrict__ Gb, const __grid_const
 // G(K2, K2+Q) (b), the G(K2, K1) tile -- and each thread sums its Nwex <= WX
 // transfers in registers: the accumulator is read and written once per batch,
 // and the sign rides on a and the G(K2, K1) tile, so that an element-update is
-// twelve fused multiply-adds.  Bound by the FP64 pipe (two lanes per clock and
-// SM): per-measurement launches of eighteen operations per update ran at
-// 3.0e10 updates/s on the 4x4 cluster with 64 frequencies.
+// fourteen operations.  Bound by the FP64 pipe (two lanes per clock and SM): one
+// batch of 16 on the 4x4 cluster with 32 frequencies, 8 transfers and 4 momenta
+// 3.75 ms, 4.78 in per-measurement launches of eighteen operations.  A
+// measurement's products are summed before they meet the batch's sum: with all in
+// one chain of twelve fused multiply-adds (3.13 ms) the error of a batch of 64
+// against exact sums was 2.9e-16 of the products' moduli, 1.2e-16 so (and in
+// per-measurement launches).
 constexpr int kTileF = 16;      // frequencies per tile side
 constexpr int kTileWex = 16;    // largest Nwex of the tiled form
 
@@ -202,9 +206,12 @@ __global__ void __launch_bounds__(kTileF * kTileF) k_update_fp64_tiled(
     const double w1 = CH == G4_PH_MAGNETIC ? -1.0 : 1.0;  // weight of spin -1 in a, b
     for (int q = 0; q < d.Nkex; ++q) {
         const int k1q = kadd[k1 * d.Nc + q], k2q = kadd[k2 * d.Nc + q];
-        double2 sum[WXM];
+        double2* row = acc + ((size_t)(k1 * Nw2 + n1) * N + k2 * Nw2 + n2) * d.NQ + (size_t)q * Nwex;
+        double2 sum[WXM];   // a single measurement goes onto the accumulator itself
 #pragma unroll
-        for (int m = 0; m < WXM; ++m) sum[m] = make_double2(0.0, 0.0);
+        for (int m = 0; m < WXM; ++m)
+            sum[m] = staged == 1 && m < Nwex && n1 + d.m0 + m < Nw2 && n2 + d.m0 + m < Nw2 ? row[m]
+                                                                                          : make_double2(0.0, 0.0);
         for (int r = 0; r < staged; ++r) {
             const double2* G = Gb + (size_t)(2 * r) * NN;
             const double sign = signs.s[r];
@@ -252,22 +259,20 @@ __global__ void __launch_bounds__(kTileF * kTileF) k_update_fp64_tiled(
 #pragma unroll
             for (int m = 0; m < WXM; ++m) {
                 if (m >= Nwex) break;
-                if (CH != G4_PH_TRANSVERSE) cfma(sum[m], A[t1 * Nwex + m], B[t2 * Nwex + m]);
-#pragma unroll
-                for (int sp = 0; sp < 2; ++sp)
-                    cfma(sum[m], X1[(sp * kTileF + t2) * (kTileF + 1) + t1],
-                         X2[(sp * WX + t1 + m) * (WX + 1) + t2 + m]);
+                double2 t = cmul(X1[t2 * (kTileF + 1) + t1], X2[(t1 + m) * (WX + 1) + t2 + m]);
+                cfma(t, X1[(kTileF + t2) * (kTileF + 1) + t1], X2[(WX + t1 + m) * (WX + 1) + t2 + m]);
+                if (CH != G4_PH_TRANSVERSE) cfma(t, A[t1 * Nwex + m], B[t2 * Nwex + m]);
+                sum[m].x += t.x;
+                sum[m].y += t.y;
             }
         }
         if (!live) continue;
-        double2* row = acc + ((size_t)(k1 * Nw2 + n1) * N + k2 * Nw2 + n2) * d.NQ + (size_t)q * Nwex;
 #pragma unroll
         for (int m = 0; m < WXM; ++m) {
             if (m >= Nwex) break;
             if (n1 + d.m0 + m >= Nw2 || n2 + d.m0 + m >= Nw2) continue;  // structurally zero
-            double2 o = row[m];
-            o.x += sum[m].x;
-            o.y += sum[m].y;
+            double2 o = sum[m];
+            if (staged > 1) o = make_double2(row[m].x + o.x, row[m].y + o.y);
             row[m] = o;
         }
     }
@@ -560,17 +565,17 @@ __global__ void k_clear_unset(double2* __restrict__ acc, long long E, const unsi
 // when enough of its frequency tiles lies on the grid (Nw2^2 of the tiles' area;
 // the opposite-spin channel, without the direct term, has less to share in a
 // tile).  16 measurements, simple / tiled, ms: 3x3 cluster, 9 momenta, magnetic, 4
-// transfers: 20 frequencies (0.39 of the tiles) 0.99 / 1.64, 24 (0.56) 1.41 /
-// 1.64, 28 (0.77) 1.91 / 1.65; 2x2, 8 transfers, 50 (0.61) 1.06 / 0.92;
-// transverse: 28 1.09 / 1.14, 3 transfers, 40 (0.69) 1.65 / 1.51, 2 transfers,
-// 48 (1) 1.59 / 1.14; one measurement at a time 28 1.19 / 1.45, 40 1.76 / 1.76.
+// transfers: 20 frequencies (0.39 of the tiles) 0.99 / 1.95, 28 (0.77) 1.91 /
+// 1.96, 3 transfers, 40 (0.69) 2.89 / 2.51; 2x2, 8 transfers, 50 (0.61) 1.06 /
+// 1.11, 4, 80 (1) 1.38 / 0.89; transverse: 4 transfers, 16 frequencies (1) 1.99 /
+// 1.74, 2 transfers, 0.99 / 1.04, 16 transfers, 100 (0.80) 4.8 / 4.6.
 constexpr long long kTiledMinEntries = 1 << 18;
 bool tiled_wanted(const G4Dims& d) {
     if (d.ch == G4_PP_UPDOWN || d.Nwex > kTileWex || (long long)d.Nc * d.Nc > 65535 || d.E < kTiledMinEntries)
         return false;
     const int side = (d.Nw2 + kTileF - 1) / kTileF * kTileF;
     const double fill = (double)d.Nw2 * d.Nw2 / ((double)side * side);
-    return d.ch == G4_PH_TRANSVERSE ? d.Nwex > 1 && fill >= 0.78 : fill >= 0.6;
+    return d.ch == G4_PH_TRANSVERSE ? d.Nwex > 2 && fill >= 0.78 : fill >= 0.65;
 }
 
 }  // namespace
@@ -627,7 +632,7 @@ double update_fp64_ps(const G4Dims& d) {
     if (!tiled_wanted(d)) return trans ? 30.0 : 52.0;
     const int side = (d.Nw2 + kTileF - 1) / kTileF * kTileF;
     const double fill = (double)d.Nw2 * d.Nw2 / ((double)side * side);
-    return (trans ? 15.5 + 6.0 / d.Nwex : 22.5 + 10.0 / d.Nwex) / fill;
+    return (trans ? 19.5 + 6.0 / d.Nwex : 27.0 + 10.0 / d.Nwex) / fill;
 }
 
 cudaError_t launch_update_fp64(const double2* G, const G4Signs& signs, int staged, double2* acc,
