@@ -93,3 +93,34 @@ def test_large_values_in_different_measurements(channel, bits):
     M[1, :, :P.N // 2] *= 2.0 ** bits
     M[2, :, P.N // 2:] *= 2.0 ** bits
     check(M, G0, np.ones(R), channel)
+
+
+def test_tiled_kernel_rounds_once_per_measurement():
+    """The plain tiled kernel against the digit sums (error below 4e-17 S here)
+    on one batch of 64 measurements.  A sum that is rounded once per measurement
+    is off by at most 2^-53 |partial sum| each time, 0.41 of it in the mean; with
+    partial sums growing evenly to S that is 0.41 x 2^-53 sqrt(64 / 3) S = 2.1e-16 S
+    over independent roundings, in the mean over the entries.  (Twelve roundings
+    per measurement, one per multiply-add, would be sqrt(12) times that bound.)"""
+    torch = cuda()
+    g4 = ensure_built()
+    p = inputs.Problem(4, 4, 16, 4, 4, 20.0, 64, 64)
+    M = torch.empty((64, 2, p.N, p.N), dtype=torch.complex128, device="cuda")
+    inputs.fill_M_device(M, seed=7)
+    G0 = torch.from_numpy(np.ascontiguousarray(inputs.g0(p))).cuda()
+    outs = []
+    for kw in ({}, dict(mem_limit=1 << 40)):     # with a memory limit: the plain kernels
+        h = g4.G4.for_problem(p, precision="fp64", **kw)
+        h.profile()
+        for r in range(64):
+            h.compute_G(M[r], G0, 1.0)
+        outs.append(h.finalize()[0])
+        assert (h.profile_read("exchange")[1] > 0) == (not kw)
+        h.close()
+    G = torch.stack([g4.build_G(M[r].contiguous(), G0) for r in range(64)])
+    ref, S = reference(p, G, np.ones(64), "ph_magnetic")
+    diag = lambda x: x.diagonal(dim1=1, dim2=2).diagonal(dim1=2, dim2=3)   # noqa: E731 n1 = n2, k1 = k2
+    err, s = diag((outs[1] - outs[0]).abs().reshape(S.shape)), diag(S)
+    rms = float(((err[s > 0] / s[s > 0]) ** 2).mean().sqrt())
+    print("rms %.2e" % rms)
+    assert rms <= 4.3e-16
