@@ -63,8 +63,8 @@
 // every time (128 x 64 x 16 per MMA: about 48 clocks of shared-memory reads for
 // 32 of arithmetic); eight accumulators of 64 columns fill tensor memory, so N
 // cannot be larger; with few values of K the epilogue.  Measured, one batch of
-// 64 on the 4x4 cluster with 64 frequencies, 8 x 16 transfers: the plain tiled
-// kernel 279 ms; here 16.6 ms (exchange 8.8, direct 2.8, packs and spread 3.4,
+// 64 on the 4x4 cluster with 64 frequencies, 8 x 16 transfers: per-measurement
+// launches of the plain tiled kernel 279 ms; here 16.6 ms (exchange 8.8, direct 2.8, packs and spread 3.4,
 // merge 1.6).  By ncu (32 frequencies) the tensor pipe is active in 65 to 71% of
 // the exchange's cycles.
 // Every wait is bounded as in the mixed path's kernels.
